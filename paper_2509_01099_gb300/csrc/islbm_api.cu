@@ -293,17 +293,28 @@ cudaError_t islbm::launch_setup_once(const void* kernel,
 
 namespace {
 
+islbm_status timed_out(Solver* s) {
+  cudaMemsetAsync(s->derr, 0, sizeof(int), s->stream);
+  return fail(s, ISLBM_ERR_TIMEOUT, "a bounded wait in the step kernel gave up");
+}
+
 // Report (and clear) a timeout recorded by a pipelined kernel.  Synchronises.
 islbm_status check_device_flag(Solver* s) {
   int flag = 0;
   cudaError_t e = cudaMemcpyAsync(&flag, s->derr, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "reading the device error flag");
-  if (flag) {
-    cudaMemsetAsync(s->derr, 0, sizeof(int), s->stream);
-    return fail(s, ISLBM_ERR_TIMEOUT, "a bounded wait in the step kernel gave up");
-  }
-  return ISLBM_OK;
+  return flag ? timed_out(s) : ISLBM_OK;
+}
+
+// Wait for a reduction launched on the handle's stream (`launch`: its launch
+// status).  The kernel leaves the sums and the error flag in pinned host memory,
+// so one synchronisation brings both.
+islbm_status reduction_result(Solver* s, cudaError_t launch) {
+  if (launch != cudaSuccess) return cuda_fail(s, launch, "launching a reduction");
+  const cudaError_t e = cudaStreamSynchronize(s->stream);
+  if (e != cudaSuccess) return cuda_fail(s, e, "waiting for a reduction");
+  return s->hresult[RED_STRIDE] != 0.0 ? timed_out(s) : ISLBM_OK;
 }
 
 islbm_status finish_reductions(Solver* s, islbm_reductions* out) {
@@ -572,7 +583,7 @@ extern "C" islbm_status islbm_create(const double* xi_x, int nx, const double* x
     tab_bytes += 2 * (((size_t)n * 16 + 255) / 256 * 256);
   }
   tab_bytes += 256;
-  s->red_blocks = 4 * 152;
+  s->red_blocks = 2 * std::max(s->sm_count, 1);
   auto cleanup = [&](islbm_status st, const std::string& m) {
     islbm_destroy(s);
     return fail(nullptr, st, m);
@@ -593,9 +604,7 @@ extern "C" islbm_status islbm_create(const double* xi_x, int nx, const double* x
   e = dmalloc(reinterpret_cast<void**>(&s->dscratch),
               (size_t)s->red_blocks * RED_STRIDE * sizeof(double));
   if (e != cudaSuccess) return cleanup(ISLBM_ERR_OOM, "islbm_create: reduction scratch");
-  e = dmalloc(reinterpret_cast<void**>(&s->dresult), RED_STRIDE * sizeof(double));
-  if (e != cudaSuccess) return cleanup(ISLBM_ERR_OOM, "islbm_create: reduction result");
-  e = cudaMallocHost(&s->hresult, RED_STRIDE * sizeof(double));
+  e = cudaMallocHost(&s->hresult, (RED_STRIDE + 1) * sizeof(double));
   if (e != cudaSuccess) return cleanup(ISLBM_ERR_OOM, "islbm_create: pinned result");
   e = dmalloc(reinterpret_cast<void**>(&s->derr), kDerrInts * sizeof(int));
   if (e != cudaSuccess) return cleanup(ISLBM_ERR_OOM, "islbm_create: error flag");
@@ -689,7 +698,6 @@ extern "C" void islbm_destroy(islbm_t s) {
   for (int b = 0; b < 2; ++b) dev_free(s->mem, s->buf[b], s->stream);
   dev_free(s->mem, s->dtables, s->stream);
   dev_free(s->mem, s->dscratch, s->stream);
-  dev_free(s->mem, s->dresult, s->stream);
   dev_free(s->mem, s->dfield, s->stream);
   dev_free(s->mem, s->derr, s->stream);
   dev_free(s->mem, s->dsnap, s->stream);
@@ -867,7 +875,7 @@ extern "C" islbm_status islbm_get_fields_device(islbm_t s, double* rho, double* 
                                                 double* v, double* w) {
   if (!s) return fail(nullptr, ISLBM_ERR_ARG, "islbm_get_fields: NULL handle");
   if (s->dim == 2 && w) return fail(s, ISLBM_ERR_ARG, "islbm_get_fields: w must be NULL in 2-D");
-  CK(s, launch_fields(*s, rho, T, u, v, w));
+  CK(s, launch_fields(*s, false, rho, T, u, v, w));
   return ISLBM_OK;
 }
 
@@ -881,7 +889,7 @@ extern "C" islbm_status islbm_get_fields(islbm_t s, double* rho, double* T, doub
   double* dst[5] = {rho, T, u, v, w};
   double* dev[5];
   for (int k = 0; k < 5; ++k) dev[k] = dst[k] ? s->dfield + k * n : nullptr;
-  CK(s, launch_fields(*s, dev[0], dev[1], dev[2], dev[3], dev[4]));
+  CK(s, launch_fields(*s, false, dev[0], dev[1], dev[2], dev[3], dev[4]));
   for (int k = 0; k < 5; ++k)
     if (dst[k])
       CK(s, cudaMemcpyAsync(dst[k], dev[k], n * 8, cudaMemcpyDeviceToHost, s->stream));
@@ -892,12 +900,6 @@ extern "C" islbm_status islbm_get_fields(islbm_t s, double* rho, double* T, doub
 // ---- time averages (FP64 accumulators on the device) ----
 
 namespace {
-__global__ void k_accumulate(double* __restrict__ acc, const double* __restrict__ src,
-                             long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    acc[i] += src[i];
-}
 __global__ void k_scale(double* __restrict__ dst, const double* __restrict__ src, double c,
                         long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -925,15 +927,9 @@ extern "C" islbm_status islbm_average_add(islbm_t s) {
     const islbm_status st = islbm_average_reset(s);
     if (st != ISLBM_OK) return st;
   }
-  islbm_status st = ensure_field_buffer(s);
-  if (st != ISLBM_OK) return st;
   const size_t n = (size_t)s->nodes;
-  // dfield holds [rho][T][u][v][w]; T, u, v (, w) are contiguous from dfield + n
-  double* f = s->dfield;
-  CK(s, launch_fields(*s, nullptr, f + n, f + 2 * n, f + 3 * n, s->dim == 3 ? f + 4 * n : nullptr));
-  const long long m = (long long)(s->dim + 1) * (long long)n;
-  k_accumulate<<<elementwise_grid(m), 256, 0, s->stream>>>(s->davg, f + n, m);
-  CK(s, cudaGetLastError());
+  double* a = s->davg;   // T, u, v (, w), one after the other
+  CK(s, launch_fields(*s, true, nullptr, a, a + n, a + 2 * n, s->dim == 3 ? a + 3 * n : nullptr));
   ++s->avg_count;
   return ISLBM_OK;
 }
@@ -980,13 +976,9 @@ extern "C" islbm_status islbm_reduce(islbm_t s, islbm_reductions* out) {
                 "islbm_reduce: the handle steps a slab; combine islbm_reduce_sums over the "
                 "slabs and finish them with islbm_finish_sums");
   {
-    const islbm_status st = check_device_flag(s);
+    const islbm_status st = reduction_result(s, launch_reduce(*s));
     if (st != ISLBM_OK) return st;
   }
-  CK(s, launch_reduce(*s));
-  CK(s, cudaMemcpyAsync(s->hresult, s->dresult, RED_STRIDE * sizeof(double),
-                        cudaMemcpyDeviceToHost, s->stream));
-  CK(s, cudaStreamSynchronize(s->stream));
   return finish_reductions(s, out);
 }
 
@@ -1000,13 +992,9 @@ extern "C" islbm_status islbm_steady_change(islbm_t s, double* du, double* dT) {
     s->snap_valid = false;
   }
   {
-    const islbm_status st = check_device_flag(s);
+    const islbm_status st = reduction_result(s, launch_steady(*s));
     if (st != ISLBM_OK) return st;
   }
-  CK(s, launch_steady(*s));
-  CK(s, cudaMemcpyAsync(s->hresult, s->dresult, RED_STRIDE * sizeof(double),
-                        cudaMemcpyDeviceToHost, s->stream));
-  CK(s, cudaStreamSynchronize(s->stream));
   const double* r = s->hresult;
   if (!s->snap_valid) {
     *du = *dT = INFINITY;
@@ -1214,13 +1202,9 @@ extern "C" islbm_status islbm_reduce_sums(islbm_t s, double* sums) {
   NvtxRange range("islbm_reduce_sums");
   if (!s || !sums) return fail(s, ISLBM_ERR_ARG, "islbm_reduce_sums: NULL argument");
   {
-    const islbm_status st = check_device_flag(s);
+    const islbm_status st = reduction_result(s, launch_reduce(*s));
     if (st != ISLBM_OK) return st;
   }
-  CK(s, launch_reduce(*s));
-  CK(s, cudaMemcpyAsync(s->hresult, s->dresult, RED_STRIDE * sizeof(double),
-                        cudaMemcpyDeviceToHost, s->stream));
-  CK(s, cudaStreamSynchronize(s->stream));
   std::memcpy(sums, s->hresult, RED_STRIDE * sizeof(double));
   return ISLBM_OK;
 }

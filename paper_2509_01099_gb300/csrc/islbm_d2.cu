@@ -20,8 +20,10 @@
 #include <type_traits>
 #include <vector>
 
+#include "islbm_exactsum.cuh"
 #include "islbm_internal.h"
 #include "islbm_lanes.cuh"
+#include "islbm_reduce.cuh"
 #include "islbm_store.cuh"
 #include "islbm_tma.cuh"
 
@@ -362,17 +364,16 @@ __global__ void k_init_pops(S* __restrict__ fout, P2<typename Store<S>::R> p,
 
 // Macroscopic state of a node from the stored post-collision deviations, in
 // FP64: rho and T are collision invariants; the collision adds F to the
-// momentum, so u = (sum e f^+ - F/2)/rho.
+// momentum, so u = (sum e f^+ - F/2)/rho = (sum e f^+)/rho - gbeta (T - T_ref)/2.
 struct NodeState {
   double rho, ux, uy, T;
 };
 
-template <typename S>
-__device__ __forceinline__ NodeState node_state(const S* __restrict__ s, size_t idx,
-                                                long long P, float aT, double gbeta, double Ts,
-                                                double Tref) {
-  typename Store<S>::R fr[9], gr[5];
-  NodeIO<S>::load(s, idx, P, aT, fr, gr);
+// The same entirely in FP64 arithmetic (FP64 storage, and states out of the
+// range of the integer sums).
+template <typename R>
+__device__ __forceinline__ NodeState node_state_fp64(const R (&fr)[9], const R (&gr)[5],
+                                                     double gbeta, double Ts, double Tref) {
   double f[9], g[5];
 #pragma unroll
   for (int i = 0; i < 9; ++i) f[i] = (double)fr[i];
@@ -391,7 +392,43 @@ __device__ __forceinline__ NodeState node_state(const S* __restrict__ s, size_t 
   return n;
 }
 
+// FP32 values (every storage form but FP64) are summed on the integer units
+// (islbm_exactsum.cuh): 7 or 8 FP64 operations a node instead of about 60 with
+// the conversions and divisions.
 template <typename S>
+__device__ __forceinline__ NodeState node_state(const S* __restrict__ s, size_t idx,
+                                                long long P, float aT, double gbeta, double Ts,
+                                                double Tref) {
+  using R = typename Store<S>::R;
+  R f[9], g[5];
+  NodeIO<S>::load(s, idx, P, aT, f, g);
+  if constexpr (std::is_same<R, float>::value) {
+    const int Ef = group_exponent(f), Eg = group_exponent(g);
+    long long F[9], G = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) F[i] = aligned(f[i], Ef);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) G += aligned(g[i], Eg);
+    const long long ax = F[1] + F[3], ay = F[2] + F[4];
+    const long long dp = F[5] - F[7], dm = F[6] - F[8], pp = F[5] + F[7], pm = F[6] + F[8];
+    NodeState n;
+    n.rho = 1.0 + aligned_to_double(F[0] + ax + ay + pp + pm, Ef);
+    if (max(Ef, Eg) < 255 && mid_range(n.rho)) {
+      const double jx = aligned_to_double(F[1] - F[3] + dp - dm, Ef);
+      const double jy = aligned_to_double(F[2] - F[4] + dp + dm, Ef);
+      const double r = quick_rcp(n.rho), h = 0.5 * gbeta;
+      n.T = aligned_to_double(G, Eg);
+      if (Ts != 0.0) n.T += Ts;
+      n.ux = jx * r;
+      n.uy = fma(jy, r, fma(-h, n.T, h * Tref));
+      return n;
+    }
+  }
+  return node_state_fp64(f, g, gbeta, Ts, Tref);
+}
+
+// ACC: add the fields to the arrays (time averages) instead of writing them.
+template <typename S, bool ACC>
 __global__ void k_fields(const S* __restrict__ s, P2<typename Store<S>::R> p, double gbeta,
                          double Ts, double Tref, double* rho, double* T, double* u, double* v) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -400,10 +437,10 @@ __global__ void k_fields(const S* __restrict__ s, P2<typename Store<S>::R> p, do
   const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, gbeta, Ts,
                                  Tref);
   const size_t node = (size_t)y * p.nx + x;
-  if (rho) rho[node] = n.rho;
-  if (T) T[node] = n.T;
-  if (u) u[node] = n.ux;
-  if (v) v[node] = n.uy;
+  if (rho) put_field<ACC>(rho + node, n.rho);
+  if (T) put_field<ACC>(T + node, n.T);
+  if (u) put_field<ACC>(u + node, n.ux);
+  if (v) put_field<ACC>(v + node, n.uy);
 }
 
 template <typename S>
@@ -453,125 +490,133 @@ __device__ __forceinline__ NodeC<typename Store<S>::R> node_state_c(
   return n;
 }
 
-// Reductions of the current state (Sec. 3, Eq. (17), Eq. (18)): per-block FP64
-// partial sums of the midpoint-rule weighted contributions of every node; the
-// nodes in the planes next to the isothermal walls and on the centre line add
-// the temperature sums from which the host finishes Eq. (17) and Nu_middle.
-// A block takes whole rows (of the slab when one is set), its threads the
-// columns.
+// Reductions of the current state (Sec. 3, Eq. (17), Eq. (18)): FP64 sums of the
+// midpoint-rule weighted contributions of every node; the nodes in the planes
+// next to the isothermal walls and on the centre line add the temperature sums
+// from which the host finishes Eq. (17) and Nu_middle.  Bound by the FP64 pipe
+// (5 operations a node: the sums over a lane's rows, weighted by W_y; W_x is
+// applied once per strip) and by the state's bytes.
 template <typename S>
-__global__ void __launch_bounds__(256)
-    k_reduce(const S* __restrict__ s, P2<typename Store<S>::R> p, double gbeta, double Ts,
-             double T0,
-             const double* __restrict__ Wx, const double* __restrict__ Wy, double* partial) {
+__global__ void __launch_bounds__(kRedThreads, 2)
+    k_reduce(const S* __restrict__ s, P2<typename Store<S>::R> p, RowStrips tk, double gbeta,
+             double Ts, double T0, const double* __restrict__ Wx, const double* __restrict__ Wy,
+             double* partial, double* out, int* words) {
   using R = typename Store<S>::R;
-  double acc[RED_COUNT];
-#pragma unroll
-  for (int k = 0; k < RED_COUNT; ++k) acc[k] = 0.0;
+  __shared__ double sh[kRedWarps][RED_STRIDE];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < RED_STRIDE) sh[warp][lane] = 0.0;
+  __syncwarp();
   const int mL = (p.nx % 2 == 0) ? p.nx / 2 - 1 : (p.nx - 1) / 2 - 1;  // left column of the centre pair
   const int mR = (p.nx % 2 == 0) ? p.nx / 2 : (p.nx + 1) / 2;           // right column
   const int mC = (p.nx % 2 == 0) ? -1 : (p.nx - 1) / 2;                  // centre column (odd n)
   const R gb = R(gbeta), ts = R(Ts), t0 = R(T0);
-  for (int y = p.y0 + (int)blockIdx.x; y < p.y1; y += (int)gridDim.x) {
-    const double wy = Wy[y];
-    for (int x = threadIdx.x; x < p.nx; x += blockDim.x) {
+  double tot[4] = {0.0, 0.0, 0.0, 0.0};   // mass, u (T - T0), |u|, |u|^2
+  R top = 0;
+  int bad = 0;
+  for (int t = blockIdx.x * kRedWarps + warp; t < tk.tasks; t += gridDim.x * kRedWarps) {
+    const int cg = t % tk.ncg, strip = t / tk.ncg;
+    const int x = cg * 32 + lane;
+    if (x >= p.nx) continue;
+    const int ya = p.y0 + strip * tk.per, yb = min(ya + tk.per, p.y0 + tk.rows);
+    const bool wall = x < 2 || x >= p.nx - 2 || x == mL || x == mR || x == mC;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, colT = 0.0;
+    for (int y = ya; y < yb; ++y) {
+      const double wy = Wy[y];
       const NodeC<R> n = node_state_c(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, gb, ts, t0);
-      const double W = Wx[x] * wy;
       const R u2 = n.ux * n.ux + n.uy * n.uy;
       const R sp = sqrt(u2);
-      const R uT = n.ux * (n.T - t0);
-      acc[RED_MASS] += W * (1.0 + (double)n.drho);
-      acc[RED_UT] += W * (double)uT;
-      acc[RED_SPEED] += W * (double)sp;
-      acc[RED_UV2] += W * (double)u2;
-      acc[RED_U2] += W * (double)u2;
-      const double T = (double)n.T;
-      if (x == 0) acc[RED_HOT1] += wy * T;
-      if (x == 1) acc[RED_HOT2] += wy * T;
-      if (x == p.nx - 1) acc[RED_COLD1] += wy * T;
-      if (x == p.nx - 2) acc[RED_COLD2] += wy * T;
-      if (x == mL) acc[RED_MIDTL] += wy * T;
-      if (x == mR) acc[RED_MIDTR] += wy * T;
-      if (mC < 0 && (x == mL || x == mR)) acc[RED_MIDCONV] += 0.5 * wy * (double)uT;
-      if (x == mC) acc[RED_MIDCONV] += wy * (double)uT;
+      acc[0] = fma(wy, 1.0 + to_d(n.drho), acc[0]);
+      acc[1] = fma(wy, to_d(n.ux * (n.T - t0)), acc[1]);
+      acc[2] = fma(wy, to_d(sp), acc[2]);
+      acc[3] = fma(wy, to_d(u2), acc[3]);
+      if (wall) colT = fma(wy, to_d(n.T), colT);
       const bool finite = isfinite(n.drho) && isfinite(n.ux) && isfinite(n.uy) && isfinite(n.T);
-      if (!finite) acc[RED_NONFINITE] += 1.0;
-      acc[RED_MAXSPEED] = fmax(acc[RED_MAXSPEED], finite ? (double)sp : 0.0);
+      bad += finite ? 0 : 1;
+      if (finite && sp > top) top = sp;
     }
-  }
-  __shared__ double sh[8][RED_COUNT];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (wall) {
+      // each of these sums belongs to one column: its lane keeps it
+      if (x == 0) sh[warp][RED_HOT1] += colT;
+      if (x == 1) sh[warp][RED_HOT2] += colT;
+      if (x == p.nx - 1) sh[warp][RED_COLD1] += colT;
+      if (x == p.nx - 2) sh[warp][RED_COLD2] += colT;
+      if (x == mL) sh[warp][RED_MIDTL] += colT;
+      if (x == mR) sh[warp][RED_MIDTR] += colT;
+      if (x == mC) sh[warp][RED_MIDCONV] += acc[1];
+      // even n: half of each of the two centre columns (RED_MIDCONV and, for
+      // the right one, the slot behind the sums, added below)
+      if (mC < 0 && x == mL) sh[warp][RED_MIDCONV] += 0.5 * acc[1];
+      if (mC < 0 && x == mR) sh[warp][RED_COUNT] += 0.5 * acc[1];
+    }
+    const double wx = Wx[x];
 #pragma unroll
-  for (int k = 0; k < RED_COUNT; ++k) {
-    const double v = (k == RED_MAXSPEED) ? warp_max(acc[k]) : warp_sum(acc[k]);
-    if (lane == 0) sh[warp][k] = v;
+    for (int k = 0; k < 4; ++k) tot[k] = fma(wx, acc[k], tot[k]);
   }
-  __syncthreads();
-  if (threadIdx.x < RED_COUNT) {
-    const int k = threadIdx.x;
-    double v = sh[0][k];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-      v = (k == RED_MAXSPEED) ? fmax(v, sh[w][k]) : v + sh[w][k];
-    partial[(size_t)blockIdx.x * RED_STRIDE + k] = v;
+  __syncwarp();
+  const double v = warp_sum4(tot);
+  bad = __reduce_add_sync(0xffffffffu, bad);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+  constexpr int slot[4] = {RED_MASS, RED_UT, RED_SPEED, RED_U2};
+  if (lane < 4) sh[warp][slot[lane]] = v;
+  if (lane == 3) sh[warp][RED_UV2] = v;
+  if (lane == 4) sh[warp][RED_NONFINITE] = (double)bad;
+  if (lane == 5) sh[warp][RED_MAXSPEED] = (double)top;
+  if (lane == 6) {
+    sh[warp][RED_MIDCONV] += sh[warp][RED_COUNT];
+    sh[warp][RED_COUNT] = 0.0;
   }
+  reduce_finish(sh, RED_MAXSPEED, partial, out, words);
 }
 
 // Steady-state criterion (Sec. 3): sum |u(t) - u(t0)|_2, sum |u(t0)|_2,
 // sum |T*(t) - T*(t0)|, sum |T*(t0)| over the nodes, against the snapshot of
 // (u, v, T*) taken at the previous check, which is then replaced by the
-// current fields.  Partial sums per block in slots 0..3 (the others zero).
-// Without a snapshot (have_snap = 0) the old values count as zero and the
-// buffer is only written.
+// current fields.  Sums in slots 0..3 (the others zero).  Without a snapshot
+// (have_snap = 0) the old values count as zero and the buffer is only written.
 template <typename S>
-__global__ void __launch_bounds__(256)
-    k_steady(const S* __restrict__ s, P2<typename Store<S>::R> p, double gbeta, double Ts,
-             double T0, double dT, int have_snap, double* snap, double* partial) {
-  double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-  const long long nodes = (long long)p.nx * p.ny;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nodes;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int y = (int)(k / p.nx), x = (int)(k - (long long)y * p.nx);
-    const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, gbeta, Ts,
-                                   T0);
-    const double Tn = (n.T - T0) / dT;
-    double ou = 0.0, ov = 0.0, oT = 0.0;
-    if (have_snap) {
-      ou = snap[k];
-      ov = snap[nodes + k];
-      oT = snap[2 * nodes + k];
-    }
-    a0 += sqrt((n.ux - ou) * (n.ux - ou) + (n.uy - ov) * (n.uy - ov));
-    a1 += sqrt(ou * ou + ov * ov);
-    a2 += fabs(Tn - oT);
-    a3 += fabs(oT);
-    snap[k] = n.ux;
-    snap[nodes + k] = n.uy;
-    snap[2 * nodes + k] = Tn;
-  }
-  __shared__ double sh[8][4];
+__global__ void __launch_bounds__(kRedThreads, 2)
+    k_steady(const S* __restrict__ s, P2<typename Store<S>::R> p, RowStrips tk, double gbeta,
+             double Ts, double T0, double dT, int have_snap, double* snap, double* partial,
+             double* out, int* words) {
+  __shared__ double sh[kRedWarps][RED_STRIDE];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3);
-  if (lane == 0) { sh[warp][0] = a0; sh[warp][1] = a1; sh[warp][2] = a2; sh[warp][3] = a3; }
-  __syncthreads();
-  if (threadIdx.x < RED_STRIDE) {
-    double v = 0.0;
-    if (threadIdx.x < 4)
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w][threadIdx.x];
-    partial[(size_t)blockIdx.x * RED_STRIDE + threadIdx.x] = v;
+  if (lane < RED_STRIDE) sh[warp][lane] = 0.0;
+  __syncwarp();
+  // after a step that gave up the snapshot stays as it is
+  const int tasks = words[0] ? 0 : tk.tasks;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  const size_t nodes = (size_t)p.nx * p.ny;
+  for (int t = blockIdx.x * kRedWarps + warp; t < tasks; t += gridDim.x * kRedWarps) {
+    const int cg = t % tk.ncg, strip = t / tk.ncg;
+    const int x = cg * 32 + lane;
+    if (x >= p.nx) continue;
+    const int ya = strip * tk.per, yb = min(ya + tk.per, tk.rows);
+    for (int y = ya; y < yb; ++y) {
+      const size_t k = (size_t)y * p.nx + x;
+      const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, gbeta,
+                                     Ts, T0);
+      const double Tn = dT == 1.0 ? n.T - T0 : (n.T - T0) / dT;
+      double ou = 0.0, ov = 0.0, oT = 0.0;
+      if (have_snap) {
+        ou = snap[k];
+        ov = snap[nodes + k];
+        oT = snap[2 * nodes + k];
+      }
+      const double du = n.ux - ou, dv = n.uy - ov;
+      a[0] += quick_sqrt(fma(du, du, dv * dv));
+      a[1] += quick_sqrt(fma(ou, ou, ov * ov));
+      a[2] += fabs(Tn - oT);
+      a[3] += fabs(oT);
+      snap[k] = n.ux;
+      snap[nodes + k] = n.uy;
+      snap[2 * nodes + k] = Tn;
+    }
   }
-}
-
-// One warp per slot sums the block partials in a fixed order (deterministic).
-__global__ void k_finish(const double* __restrict__ partial, int blocks, double* out) {
-  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (k >= RED_COUNT) return;
-  double v = 0.0;
-  for (int b = lane; b < blocks; b += 32) {
-    const double x = partial[(size_t)b * RED_STRIDE + k];
-    v = (k == RED_MAXSPEED) ? fmax(v, x) : v + x;
-  }
-  v = (k == RED_MAXSPEED) ? warp_max(v) : warp_sum(v);
-  if (lane == 0) out[k] = v;
+  __syncwarp();
+  const double v = warp_sum4(a);
+  if (lane < 4) sh[warp][lane] = v;
+  reduce_finish(sh, -1, partial, out, words);
 }
 
 template <typename R>
@@ -1519,11 +1564,11 @@ struct InitPopsFn {
 
 template <typename S>
 struct FieldsFn {
-  static cudaError_t run(Solver& s, double* rho, double* T, double* u, double* v) {
+  static cudaError_t run(Solver& s, bool acc, double* rho, double* T, double* u, double* v) {
     using R = typename Store<S>::R;
-    k_fields<S><<<grid2(s), block2(), 0, s.stream>>>(static_cast<const S*>(s.buf[s.cur]),
-                                                    make_params<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0, rho,
-                                                    T, u, v);
+    const auto k = acc ? k_fields<S, true> : k_fields<S, false>;
+    k<<<grid2(s), block2(), 0, s.stream>>>(static_cast<const S*>(s.buf[s.cur]), make_params<R>(s),
+                                           s.ph.gbeta, s.ph.Ts, s.ph.T0, rho, T, u, v);
     return cudaGetLastError();
   }
 };
@@ -1542,9 +1587,10 @@ template <typename S>
 struct ReduceFn {
   static cudaError_t run(Solver& s) {
     using R = typename Store<S>::R;
-    k_reduce<S><<<s.red_blocks, 256, 0, s.stream>>>(
-        static_cast<const S*>(s.buf[s.cur]), make_params<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0,
-        s.dax[0].W, s.dax[1].W, s.dscratch);
+    const RowStrips tk = row_strips(s.n[0], step_rows(s), s.red_blocks);
+    k_reduce<S><<<tk.blocks, kRedThreads, 0, s.stream>>>(
+        static_cast<const S*>(s.buf[s.cur]), make_params<R>(s), tk, s.ph.gbeta, s.ph.Ts, s.ph.T0,
+        s.dax[0].W, s.dax[1].W, s.dscratch, s.hresult, s.derr);
     return cudaGetLastError();
   }
 };
@@ -1553,9 +1599,10 @@ template <typename S>
 struct SteadyFn {
   static cudaError_t run(Solver& s) {
     using R = typename Store<S>::R;
-    k_steady<S><<<s.red_blocks, 256, 0, s.stream>>>(
-        static_cast<const S*>(s.buf[s.cur]), make_params<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0,
-        s.ph.dT, s.snap_valid ? 1 : 0, s.dsnap, s.dscratch);
+    const RowStrips tk = row_strips(s.n[0], s.n[1], s.red_blocks);
+    k_steady<S><<<tk.blocks, kRedThreads, 0, s.stream>>>(
+        static_cast<const S*>(s.buf[s.cur]), make_params<R>(s), tk, s.ph.gbeta, s.ph.Ts, s.ph.T0,
+        s.ph.dT, s.snap_valid ? 1 : 0, s.dsnap, s.dscratch, s.hresult, s.derr);
     return cudaGetLastError();
   }
 };
@@ -1580,10 +1627,10 @@ cudaError_t launch_init_populations(Solver& s, const double* f, const double* g)
   return dispatch<InitPopsFn>(s, f, g);
 }
 
-cudaError_t launch_fields(Solver& s, double* rho, double* T, double* u0, double* u1,
+cudaError_t launch_fields(Solver& s, bool acc, double* rho, double* T, double* u0, double* u1,
                           double* u2) {
-  if (s.dim == 3) return launch_fields_3d(s, rho, T, u0, u1, u2);
-  return dispatch<FieldsFn>(s, rho, T, u0, u1);
+  if (s.dim == 3) return launch_fields_3d(s, acc, rho, T, u0, u1, u2);
+  return dispatch<FieldsFn>(s, acc, rho, T, u0, u1);
 }
 
 cudaError_t launch_populations(Solver& s, double* f, double* g) {
@@ -1592,20 +1639,11 @@ cudaError_t launch_populations(Solver& s, double* f, double* g) {
 }
 
 cudaError_t launch_reduce(Solver& s) {
-  cudaError_t e = (s.dim == 3) ? launch_reduce_3d(s) : dispatch<ReduceFn>(s);
-  if (e != cudaSuccess) return e;
-  return launch_finish_reduce(s);
+  return s.dim == 3 ? launch_reduce_3d(s) : dispatch<ReduceFn>(s);
 }
 
 cudaError_t launch_steady(Solver& s) {
-  cudaError_t e = (s.dim == 3) ? launch_steady_3d(s) : dispatch<SteadyFn>(s);
-  if (e != cudaSuccess) return e;
-  return launch_finish_reduce(s);
-}
-
-cudaError_t launch_finish_reduce(Solver& s) {
-  k_finish<<<1, 32 * RED_COUNT, 0, s.stream>>>(s.dscratch, s.red_blocks, s.dresult);
-  return cudaGetLastError();
+  return s.dim == 3 ? launch_steady_3d(s) : dispatch<SteadyFn>(s);
 }
 
 // ---- batched step ----

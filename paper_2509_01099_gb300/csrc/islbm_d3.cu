@@ -10,7 +10,12 @@
 // pull (interpolated virtual streaming or wall rule) -> macroscopic moments ->
 // MRT collision -> store.  Hot wall at x = 0, cold wall at x = 1, the y and z
 // walls adiabatic; gravity along -y.
+#include <algorithm>
+#include <type_traits>
+
+#include "islbm_exactsum.cuh"
 #include "islbm_internal.h"
+#include "islbm_reduce.cuh"
 #include "islbm_store.cuh"
 #include "islbm_d3_common.cuh"
 
@@ -198,26 +203,60 @@ struct NodeState3 {
   double rho, ux, uy, uz, T;
 };
 
+// Sums of a node's deviations and their first moments, in any arithmetic type
+// that adds: rho - 1, j and T - T_s.
+template <typename V>
+__device__ __forceinline__ void sums3(const V (&f)[19], const V (&g)[7], V& drho, V& jx, V& jy,
+                                      V& jz, V& Tr) {
+  const V xyp = f[7] + f[8], xym = f[9] + f[10], xzp = f[11] + f[12], xzm = f[13] + f[14];
+  const V yzp = f[15] + f[16], yzm = f[17] + f[18];
+  drho = (f[0] + ((f[1] + f[2]) + (f[3] + f[4]) + (f[5] + f[6]))) +
+         ((xyp + xym) + (xzp + xzm) + (yzp + yzm));
+  const V a = f[7] - f[8], b = f[9] - f[10], c = f[11] - f[12], d = f[13] - f[14];
+  const V e = f[15] - f[16], h = f[17] - f[18];
+  jx = (f[1] - f[2]) + (a + b) + (c + d);
+  jy = (f[3] - f[4]) + (a - b) + (e + h);
+  jz = (f[5] - f[6]) + (c - d) + (e - h);
+  Tr = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + g[6]);
+}
+
+// As the 2-D node_state: FP32 values are summed on the integer units.
 template <typename S>
 __device__ __forceinline__ NodeState3 node_state3(const S* __restrict__ s, size_t idx,
                                                   long long P, double gbeta, double Ts,
                                                   double Tref) {
-  double f[19], g[7];
+  using R = typename Store<S>::R;
+  R fr[19], gr[7];
 #pragma unroll
-  for (int i = 0; i < 19; ++i) f[i] = (double)Store<S>::ld(s + i * P + idx);
+  for (int i = 0; i < 19; ++i) fr[i] = Store<S>::ld(s + i * P + idx);
 #pragma unroll
-  for (int i = 0; i < 7; ++i) g[i] = (double)Store<S>::ld(s + (19 + i) * P + idx);
-  double drho = 0, jx = 0, jy = 0, jz = 0, Tr = 0;
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    drho += f[i];
-    jx += kE3[i][0] * f[i];
-    jy += kE3[i][1] * f[i];
-    jz += kE3[i][2] * f[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 7; ++i) Tr += g[i];
+  for (int i = 0; i < 7; ++i) gr[i] = Store<S>::ld(s + (19 + i) * P + idx);
   NodeState3 n;
+  if constexpr (std::is_same<R, float>::value) {
+    const int Ef = group_exponent(fr), Eg = group_exponent(gr);
+    long long F[19], G[7], M, X, Y, Z, Q;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) F[i] = aligned(fr[i], Ef);
+#pragma unroll
+    for (int i = 0; i < 7; ++i) G[i] = aligned(gr[i], Eg);
+    sums3(F, G, M, X, Y, Z, Q);
+    n.rho = 1.0 + aligned_to_double(M, Ef);
+    if (max(Ef, Eg) < 255 && mid_range(n.rho)) {
+      const double r = quick_rcp(n.rho), h = 0.5 * gbeta;
+      n.T = aligned_to_double(Q, Eg);
+      if (Ts != 0.0) n.T += Ts;
+      n.ux = aligned_to_double(X, Ef) * r;
+      n.uy = fma(aligned_to_double(Y, Ef), r, fma(-h, n.T, h * Tref));
+      n.uz = aligned_to_double(Z, Ef) * r;
+      return n;
+    }
+  }
+  double f[19], g[7], drho, jx, jy, jz, Tr;
+#pragma unroll
+  for (int i = 0; i < 19; ++i) f[i] = (double)fr[i];
+#pragma unroll
+  for (int i = 0; i < 7; ++i) g[i] = (double)gr[i];
+  sums3(f, g, drho, jx, jy, jz, Tr);
   n.rho = 1.0 + drho;
   n.T = Tr + Ts;
   const double Fy = n.rho * gbeta * (n.T - Tref);
@@ -227,7 +266,8 @@ __device__ __forceinline__ NodeState3 node_state3(const S* __restrict__ s, size_
   return n;
 }
 
-template <typename S>
+// ACC: add the fields to the arrays (time averages) instead of writing them.
+template <typename S, bool ACC>
 __global__ void k_fields3(const S* __restrict__ s, P3<typename Store<S>::R> p, double gbeta,
                           double Ts, double Tref, double* rho, double* T, double* u, double* v,
                           double* w) {
@@ -238,11 +278,11 @@ __global__ void k_fields3(const S* __restrict__ s, P3<typename Store<S>::R> p, d
   const NodeState3 n =
       node_state3(s, ((size_t)z * p.ny + y) * p.pitch + x, p.plane, gbeta, Ts, Tref);
   const size_t node = ((size_t)z * p.ny + y) * p.nx + x;
-  if (rho) rho[node] = n.rho;
-  if (T) T[node] = n.T;
-  if (u) u[node] = n.ux;
-  if (v) v[node] = n.uy;
-  if (w) w[node] = n.uz;
+  if (rho) put_field<ACC>(rho + node, n.rho);
+  if (T) put_field<ACC>(T + node, n.T);
+  if (u) put_field<ACC>(u + node, n.ux);
+  if (v) put_field<ACC>(v + node, n.uy);
+  if (w) put_field<ACC>(w + node, n.uz);
 }
 
 template <typename S>
@@ -280,16 +320,8 @@ __device__ __forceinline__ NodeC3<typename Store<S>::R> node_state3_c(
   for (int i = 0; i < 19; ++i) f[i] = Store<S>::ld(s + i * P + idx);
 #pragma unroll
   for (int i = 0; i < 7; ++i) g[i] = Store<S>::ld(s + (19 + i) * P + idx);
-  R drho = 0, jx = 0, jy = 0, jz = 0, Tr = 0;
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    drho += f[i];
-    jx += R(kE3[i][0]) * f[i];
-    jy += R(kE3[i][1]) * f[i];
-    jz += R(kE3[i][2]) * f[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 7; ++i) Tr += g[i];
+  R drho, jx, jy, jz, Tr;
+  sums3(f, g, drho, jx, jy, jz, Tr);
   NodeC3<R> n;
   n.drho = drho;
   const R rho = R(1) + drho;
@@ -302,105 +334,120 @@ __device__ __forceinline__ NodeC3<typename Store<S>::R> node_state3_c(
 }
 
 // Reductions (Sec. 4): FP64 volume sums and the wall-plane temperature sums of
-// Eq. (17) with the wall-plane weights W_y W_z.  A block takes whole rows
-// (y, z), its threads the columns.
+// Eq. (17) with the wall-plane weights W_y W_z; the work is dealt as in the 2-D
+// kernel, a row being one (y, z) line.
 template <typename S>
-__global__ void __launch_bounds__(256)
-    k_reduce3(const S* __restrict__ s, P3<typename Store<S>::R> p, double gbeta, double Ts,
-              double T0,
-              const double* __restrict__ Wx, const double* __restrict__ Wy,
-              const double* __restrict__ Wz, double* partial) {
+__global__ void __launch_bounds__(kRedThreads, 2)
+    k_reduce3(const S* __restrict__ s, P3<typename Store<S>::R> p, RowStrips tk, double gbeta,
+              double Ts, double T0, const double* __restrict__ Wx, const double* __restrict__ Wy,
+              const double* __restrict__ Wz, double* partial, double* out, int* words) {
   using R = typename Store<S>::R;
-  double acc[RED_COUNT];
-#pragma unroll
-  for (int k = 0; k < RED_COUNT; ++k) acc[k] = 0.0;
-  const int rows = p.ny * p.nz;
+  __shared__ double sh[kRedWarps][RED_STRIDE];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < RED_STRIDE) sh[warp][lane] = 0.0;
+  __syncwarp();
   const R gb = R(gbeta), ts = R(Ts), t0 = R(T0);
-  for (int row = (int)blockIdx.x; row < rows; row += (int)gridDim.x) {
-    const int z = row / p.ny, y = row - z * p.ny;
-    const double wp = Wy[y] * Wz[z];
-    const size_t base = ((size_t)z * p.ny + y) * p.pitch;
-    for (int x = threadIdx.x; x < p.nx; x += blockDim.x) {
-      const NodeC3<R> n = node_state3_c(s, base + x, p.plane, gb, ts, t0);
-      const double W = Wx[x] * wp;
+  double tot[4] = {0.0, 0.0, 0.0, 0.0};   // mass, u (T - T0), |u|, |u|^2
+  double uv = 0.0;                        // u^2 + v^2
+  R top = 0;
+  int bad = 0;
+  for (int t = blockIdx.x * kRedWarps + warp; t < tk.tasks; t += gridDim.x * kRedWarps) {
+    const int cg = t % tk.ncg, strip = t / tk.ncg;
+    const int x = cg * 32 + lane;
+    if (x >= p.nx) continue;
+    const int ra = strip * tk.per, rb = min(ra + tk.per, tk.rows);
+    const bool wall = x < 2 || x >= p.nx - 2;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, auv = 0.0, colT = 0.0;
+    int z = ra / p.ny, y = ra - z * p.ny;
+    for (int row = ra; row < rb; ++row) {
+      const double wp = Wy[y] * Wz[z];
+      const NodeC3<R> n = node_state3_c(s, (size_t)row * p.pitch + x, p.plane, gb, ts, t0);
       const R uv2 = n.ux * n.ux + n.uy * n.uy;
       const R u2 = uv2 + n.uz * n.uz;
       const R sp = sqrt(u2);
-      acc[RED_MASS] += W * (1.0 + (double)n.drho);
-      acc[RED_UT] += W * (double)(n.ux * (n.T - t0));
-      acc[RED_SPEED] += W * (double)sp;
-      acc[RED_UV2] += W * (double)uv2;
-      acc[RED_U2] += W * (double)u2;
-      const double T = (double)n.T;
-      if (x == 0) acc[RED_HOT1] += wp * T;
-      if (x == 1) acc[RED_HOT2] += wp * T;
-      if (x == p.nx - 1) acc[RED_COLD1] += wp * T;
-      if (x == p.nx - 2) acc[RED_COLD2] += wp * T;
+      acc[0] = fma(wp, 1.0 + to_d(n.drho), acc[0]);
+      acc[1] = fma(wp, to_d(n.ux * (n.T - t0)), acc[1]);
+      acc[2] = fma(wp, to_d(sp), acc[2]);
+      acc[3] = fma(wp, to_d(u2), acc[3]);
+      auv = fma(wp, to_d(uv2), auv);
+      if (wall) colT = fma(wp, to_d(n.T), colT);
       const bool finite = isfinite(n.drho) && isfinite(n.ux) && isfinite(n.uy) &&
                           isfinite(n.uz) && isfinite(n.T);
-      if (!finite) acc[RED_NONFINITE] += 1.0;
-      acc[RED_MAXSPEED] = fmax(acc[RED_MAXSPEED], finite ? (double)sp : 0.0);
+      bad += finite ? 0 : 1;
+      if (finite && sp > top) top = sp;
+      if (++y == p.ny) {
+        y = 0;
+        ++z;
+      }
     }
-  }
-  __shared__ double sh[8][RED_COUNT];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (x == 0) sh[warp][RED_HOT1] += colT;
+    if (x == 1) sh[warp][RED_HOT2] += colT;
+    if (x == p.nx - 1) sh[warp][RED_COLD1] += colT;
+    if (x == p.nx - 2) sh[warp][RED_COLD2] += colT;
+    const double wx = Wx[x];
 #pragma unroll
-  for (int k = 0; k < RED_COUNT; ++k) {
-    const double v = (k == RED_MAXSPEED) ? warp_max(acc[k]) : warp_sum(acc[k]);
-    if (lane == 0) sh[warp][k] = v;
+    for (int k = 0; k < 4; ++k) tot[k] = fma(wx, acc[k], tot[k]);
+    uv = fma(wx, auv, uv);
   }
-  __syncthreads();
-  if (threadIdx.x < RED_COUNT) {
-    const int k = threadIdx.x;
-    double v = sh[0][k];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-      v = (k == RED_MAXSPEED) ? fmax(v, sh[w][k]) : v + sh[w][k];
-    partial[(size_t)blockIdx.x * RED_STRIDE + k] = v;
-  }
+  __syncwarp();
+  const double v = warp_sum4(tot);
+  uv = warp_sum(uv);
+  bad = __reduce_add_sync(0xffffffffu, bad);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+  constexpr int slot[4] = {RED_MASS, RED_UT, RED_SPEED, RED_U2};
+  if (lane < 4) sh[warp][slot[lane]] = v;
+  if (lane == 4) sh[warp][RED_UV2] = uv;
+  if (lane == 5) sh[warp][RED_NONFINITE] = (double)bad;
+  if (lane == 6) sh[warp][RED_MAXSPEED] = (double)top;
+  reduce_finish(sh, RED_MAXSPEED, partial, out, words);
 }
 
 // Steady-state criterion (Sec. 3) in 3-D, as the 2-D kernel with (u, v, w, T*).
 template <typename S>
-__global__ void __launch_bounds__(256)
-    k_steady3(const S* __restrict__ s, P3<typename Store<S>::R> p, double gbeta, double Ts,
-              double T0, double dT, int have_snap, double* snap, double* partial) {
-  double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-  const long long nodes = (long long)p.nx * p.ny * p.nz;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < nodes;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(k % p.nx);
-    const long long r = k / p.nx;
-    const int y = (int)(r % p.ny), z = (int)(r / p.ny);
-    const NodeState3 n =
-        node_state3(s, ((size_t)z * p.ny + y) * p.pitch + x, p.plane, gbeta, Ts, T0);
-    const double Tn = (n.T - T0) / dT;
-    double ou = 0.0, ov = 0.0, ow = 0.0, oT = 0.0;
-    if (have_snap) {
-      ou = snap[k];
-      ov = snap[nodes + k];
-      ow = snap[2 * nodes + k];
-      oT = snap[3 * nodes + k];
-    }
-    a0 += sqrt((n.ux - ou) * (n.ux - ou) + (n.uy - ov) * (n.uy - ov) + (n.uz - ow) * (n.uz - ow));
-    a1 += sqrt(ou * ou + ov * ov + ow * ow);
-    a2 += fabs(Tn - oT);
-    a3 += fabs(oT);
-    snap[k] = n.ux;
-    snap[nodes + k] = n.uy;
-    snap[2 * nodes + k] = n.uz;
-    snap[3 * nodes + k] = Tn;
-  }
-  __shared__ double sh[8][4];
+__global__ void __launch_bounds__(kRedThreads, 2)
+    k_steady3(const S* __restrict__ s, P3<typename Store<S>::R> p, RowStrips tk, double gbeta,
+              double Ts, double T0, double dT, int have_snap, double* snap, double* partial,
+              double* out, int* words) {
+  __shared__ double sh[kRedWarps][RED_STRIDE];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3);
-  if (lane == 0) { sh[warp][0] = a0; sh[warp][1] = a1; sh[warp][2] = a2; sh[warp][3] = a3; }
-  __syncthreads();
-  if (threadIdx.x < RED_STRIDE) {
-    double v = 0.0;
-    if (threadIdx.x < 4)
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w][threadIdx.x];
-    partial[(size_t)blockIdx.x * RED_STRIDE + threadIdx.x] = v;
+  if (lane < RED_STRIDE) sh[warp][lane] = 0.0;
+  __syncwarp();
+  // after a step that gave up the snapshot stays as it is
+  const int tasks = words[0] ? 0 : tk.tasks;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  const size_t nodes = (size_t)p.nx * p.ny * p.nz;
+  for (int t = blockIdx.x * kRedWarps + warp; t < tasks; t += gridDim.x * kRedWarps) {
+    const int cg = t % tk.ncg, strip = t / tk.ncg;
+    const int x = cg * 32 + lane;
+    if (x >= p.nx) continue;
+    const int ra = strip * tk.per, rb = min(ra + tk.per, tk.rows);
+    for (int row = ra; row < rb; ++row) {
+      const size_t k = (size_t)row * p.nx + x;
+      const NodeState3 n = node_state3(s, (size_t)row * p.pitch + x, p.plane, gbeta, Ts, T0);
+      const double Tn = dT == 1.0 ? n.T - T0 : (n.T - T0) / dT;
+      double ou = 0.0, ov = 0.0, ow = 0.0, oT = 0.0;
+      if (have_snap) {
+        ou = snap[k];
+        ov = snap[nodes + k];
+        ow = snap[2 * nodes + k];
+        oT = snap[3 * nodes + k];
+      }
+      const double du = n.ux - ou, dv = n.uy - ov, dw = n.uz - ow;
+      a[0] += quick_sqrt(fma(du, du, fma(dv, dv, dw * dw)));
+      a[1] += quick_sqrt(fma(ou, ou, fma(ov, ov, ow * ow)));
+      a[2] += fabs(Tn - oT);
+      a[3] += fabs(oT);
+      snap[k] = n.ux;
+      snap[nodes + k] = n.uy;
+      snap[2 * nodes + k] = n.uz;
+      snap[3 * nodes + k] = Tn;
+    }
   }
+  __syncwarp();
+  const double v = warp_sum4(a);
+  if (lane < 4) sh[warp][lane] = v;
+  reduce_finish(sh, -1, partial, out, words);
 }
 
 dim3 block3() { return dim3(32, 8, 1); }
@@ -455,11 +502,13 @@ struct InitPops3 {
 
 template <typename S>
 struct Fields3 {
-  static cudaError_t run(Solver& s, double* rho, double* T, double* u, double* v, double* w) {
+  static cudaError_t run(Solver& s, bool acc, double* rho, double* T, double* u, double* v,
+                         double* w) {
     using R = typename Store<S>::R;
-    k_fields3<S><<<grid3(s), block3(), 0, s.stream>>>(static_cast<const S*>(s.buf[s.cur]),
-                                                     make_params3<R>(s), s.ph.gbeta, s.ph.Ts,
-                                                     s.ph.T0, rho, T, u, v, w);
+    const auto k = acc ? k_fields3<S, true> : k_fields3<S, false>;
+    k<<<grid3(s), block3(), 0, s.stream>>>(static_cast<const S*>(s.buf[s.cur]),
+                                           make_params3<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0, rho,
+                                           T, u, v, w);
     return cudaGetLastError();
   }
 };
@@ -478,9 +527,10 @@ template <typename S>
 struct Reduce3 {
   static cudaError_t run(Solver& s) {
     using R = typename Store<S>::R;
-    k_reduce3<S><<<s.red_blocks, 256, 0, s.stream>>>(
-        static_cast<const S*>(s.buf[s.cur]), make_params3<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0,
-        s.dax[0].W, s.dax[1].W, s.dax[2].W, s.dscratch);
+    const RowStrips tk = row_strips(s.n[0], (long long)s.n[1] * s.n[2], s.red_blocks);
+    k_reduce3<S><<<tk.blocks, kRedThreads, 0, s.stream>>>(
+        static_cast<const S*>(s.buf[s.cur]), make_params3<R>(s), tk, s.ph.gbeta, s.ph.Ts, s.ph.T0,
+        s.dax[0].W, s.dax[1].W, s.dax[2].W, s.dscratch, s.hresult, s.derr);
     return cudaGetLastError();
   }
 };
@@ -489,9 +539,10 @@ template <typename S>
 struct Steady3 {
   static cudaError_t run(Solver& s) {
     using R = typename Store<S>::R;
-    k_steady3<S><<<s.red_blocks, 256, 0, s.stream>>>(
-        static_cast<const S*>(s.buf[s.cur]), make_params3<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0,
-        s.ph.dT, s.snap_valid ? 1 : 0, s.dsnap, s.dscratch);
+    const RowStrips tk = row_strips(s.n[0], (long long)s.n[1] * s.n[2], s.red_blocks);
+    k_steady3<S><<<tk.blocks, kRedThreads, 0, s.stream>>>(
+        static_cast<const S*>(s.buf[s.cur]), make_params3<R>(s), tk, s.ph.gbeta, s.ph.Ts, s.ph.T0,
+        s.ph.dT, s.snap_valid ? 1 : 0, s.dsnap, s.dscratch, s.hresult, s.derr);
     return cudaGetLastError();
   }
 };
@@ -515,9 +566,9 @@ cudaError_t launch_init_populations_3d(Solver& s, const double* f, const double*
   return dispatch3<InitPops3>(s, f, g);
 }
 
-cudaError_t launch_fields_3d(Solver& s, double* rho, double* T, double* u0, double* u1,
+cudaError_t launch_fields_3d(Solver& s, bool acc, double* rho, double* T, double* u0, double* u1,
                              double* u2) {
-  return dispatch3<Fields3>(s, rho, T, u0, u1, u2);
+  return dispatch3<Fields3>(s, acc, rho, T, u0, u1, u2);
 }
 
 cudaError_t launch_populations_3d(Solver& s, double* f, double* g) {

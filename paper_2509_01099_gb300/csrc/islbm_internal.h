@@ -150,10 +150,9 @@ struct Solver {
   Axis ax[3];
   void* dtables = nullptr;
   DevAxis dax[3]{};
-  double* dscratch = nullptr;     // reduction partials [blocks][RED_COUNT]
+  double* dscratch = nullptr;     // reduction partials [blocks][RED_STRIDE]
   int red_blocks = 0;
-  double* dresult = nullptr;      // finished reduction vector
-  double* hresult = nullptr;      // pinned host copy
+  double* hresult = nullptr;      // finished reduction vector and error flag (pinned host memory)
   double* dfield = nullptr;       // staging for field upload / download (5 * nodes)
   double* dsnap = nullptr;        // steady-state snapshot (u, v[, w], T*), allocated on first use
   double* davg = nullptr;         // time-average accumulators (T, u, v[, w]), FP64
@@ -167,8 +166,9 @@ struct Solver {
   // [row_begin, row_end) only (row_end == 0: every row)
   int row_begin = 0, row_end = 0;
   int sm_count = 0;
-  // device words of the pipelined kernels: [0] error flag, [1] tiles claimed,
-  // [2] CTAs finished (the 2-D TMA kernel's dynamic schedule; zero between launches)
+  // device words of the kernels: [0] error flag, [1] tiles claimed, [2] CTAs
+  // finished (the 2-D TMA kernel's dynamic schedule), [3] blocks of a reduction
+  // finished ([1] to [3] are zero between launches)
   int* derr = nullptr;
   alignas(128) unsigned char tmap[2][128];   // TMA descriptors of buf[0] / buf[1]
   alignas(128) unsigned char tmap_m[2][128]; // FP16NEQ: of their moment planes
@@ -192,11 +192,14 @@ cudaError_t launch_init_fields(Solver& s, const double* rho, const double* T, co
 cudaError_t launch_init_populations(Solver& s, const double* f, const double* g);
 // One fused step: buf[cur] -> buf[cur ^ 1].
 cudaError_t launch_step(Solver& s);
-// Macroscopic fields of the current state into device arrays (any may be null).
-cudaError_t launch_fields(Solver& s, double* rho, double* T, double* u0, double* u1, double* u2);
+// Macroscopic fields of the current state into device arrays (any may be null);
+// accumulate: added to the arrays.
+cudaError_t launch_fields(Solver& s, bool accumulate, double* rho, double* T, double* u0,
+                          double* u1, double* u2);
 // Full FP64 post-collision populations of the current state, [q][node] device arrays.
 cudaError_t launch_populations(Solver& s, double* f, double* g);
-// Reductions of the current state into s.dresult (RED_COUNT doubles).
+// Reductions of the current state into s.hresult: RED_COUNT sums and, at
+// RED_STRIDE, the step kernels' error flag (valid once the stream is idle).
 cudaError_t launch_reduce(Solver& s);
 
 cudaError_t launch_init_fields_3d(Solver& s, const double* rho, const double* T,
@@ -219,14 +222,13 @@ int step_3d_zm_box(int elem, int variant, int g, unsigned (&box)[5]);
 int step_3d_zm_first_plane(int g);
 int step_3d_zm_split(int g);
 inline bool is_zm3d(int variant) { return variant == KV_ZM3D || variant == KV_ZM3D_T4; }
-cudaError_t launch_fields_3d(Solver& s, double* rho, double* T, double* u0, double* u1,
-                             double* u2);
+cudaError_t launch_fields_3d(Solver& s, bool accumulate, double* rho, double* T, double* u0,
+                             double* u1, double* u2);
 cudaError_t launch_populations_3d(Solver& s, double* f, double* g);
 cudaError_t launch_reduce_3d(Solver& s);
 
-// Deterministic final sum of the per-block partials (islbm_d2.cu).
-cudaError_t launch_finish_reduce(Solver& s);
-// Steady-state sums against the snapshot (which is then refreshed); slots 0..3 of dresult.
+// Steady-state sums against the snapshot (which is then refreshed); slots 0..3 of
+// hresult, and the error flag as launch_reduce.
 cudaError_t launch_steady(Solver& s);
 cudaError_t launch_steady_3d(Solver& s);
 
