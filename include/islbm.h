@@ -431,6 +431,40 @@ ISLBM_API islbm_status islbm_cnn_adam(float* w, void* wb, const float* g, float*
                                       long long n, float lr, float beta1, float beta2,
                                       float eps, long long t, void* stream);
 
+/* The whole network, its layers fused (convolutions without an im2col copy).
+ * channels[stages + 1]: input channels of each convolution, then the output's;
+ * stage s upsamples 2x, convolves 3x3 and applies tanh, the last one only
+ * convolves.  params: W1 [16][hidden], b1, W2 [hidden][base^2 channels[0]], b2,
+ * then Wc_s [>= 9 channels[s]][channels[s + 1]], bc_s of every stage; weights
+ * bf16, biases FP32.  z: batch x 16 features in HOST memory (read before the
+ * call returns).  Written: zk [batch][16] (the features rounded to bf16; may be
+ * NULL), h1 [batch][hidden], acts[0 .. stages]: the second layer's output and
+ * every stage's.  acts 16-byte aligned.  Limits: 64 channels, 8 stages, 512
+ * hidden units, 256 x 256 outputs (a wide layer fewer,
+ * by its shared memory); ISLBM_ERR_ARG beyond them. */
+ISLBM_API islbm_status islbm_cnn_forward(int stages, const int* channels, int base, int hidden,
+                                         const void* const* params, const float* z, int batch,
+                                         float* zk, float* h1, float* const* acts, void* stream);
+/* Bytes of scratch that islbm_cnn_backward needs (on the current device). */
+ISLBM_API islbm_status islbm_cnn_backward_scratch(int stages, const int* channels, int base,
+                                                  int hidden, int batch,
+                                                  unsigned long long* bytes);
+/* Gradients of all parameters (in the order of params, FP32; the rows of Wc_s
+ * between 9 channels[s] and the next multiple of 16 are set to zero) for the
+ * output gradient dy.  zk, h1 and acts are those of the forward call, scratch
+ * is 256-byte aligned.  Sums run in a fixed order: the same bits on every run. */
+ISLBM_API islbm_status islbm_cnn_backward(int stages, const int* channels, int base, int hidden,
+                                          const void* const* params, int batch, const float* zk,
+                                          const float* h1, const float* const* acts,
+                                          const float* dy, float* const* grads, float* scratch,
+                                          void* stream);
+/* islbm_cnn_adam of `tensors` tensors at once (wb[k] may be NULL). */
+ISLBM_API islbm_status islbm_cnn_adam_all(int tensors, float* const* w, void* const* wb,
+                                          const float* const* g, float* const* m,
+                                          float* const* v, const long long* n, float lr,
+                                          float beta1, float beta2, float eps, long long t,
+                                          void* stream);
+
 /* Solver fields <-> network channels for `nodes` nodes (the 2-D node order of
  * islbm_get_fields_device): y[3k..3k+2] = ((T - T_mid) / T_scale,
  * u / u_scale, v / u_scale) with T, u, v FP64 device arrays and y FP32 NHWC;

@@ -12,10 +12,11 @@ Architecture (about 1.1M parameters at the default size):
     for each stage: up 2x, 3x3 conv, tanh       channels C1 .. Cs
     y = 3x3 conv (no activation)                 3 channels: T* - 1/2, s u*, s v*
 
-Every operation runs in the library's CUDA kernels (islbm_cnn_*): BF16
-tensor-core GEMMs with FP32 accumulation for the fully connected layers and
-the im2col convolutions, and elementwise kernels.  torch supplies device
-memory and the stream only.
+Every operation runs in the library's CUDA kernels: BF16 tensor-core products
+with FP32 accumulation.  Networks of up to 64 channels run as fused layers
+(islbm_cnn_forward / _backward), wider ones as a chain of GEMMs on im2col
+copies and elementwise kernels.  torch supplies device memory and the stream
+only.
 """
 from __future__ import annotations
 
@@ -42,6 +43,10 @@ def features(log10_ra, pr, a):
 def _ck(st):
     if st != 0:
         raise IslbmError(st, "warm-start network kernel")
+
+
+def _ptrs(tensors):
+    return (ctypes.c_void_p * len(tensors))(*[None if t is None else t.data_ptr() for t in tensors])
 
 
 def _p(t):
@@ -86,6 +91,12 @@ class WarmStartNet:
             if name.startswith("W"):
                 self.bf[name] = torch.empty(shp, dtype=torch.bfloat16, device=device)
                 self._to_bf16(self.params[name], self.bf[name])
+        stages = list(self.channels) + [out_ch]
+        self._chan = (ctypes.c_int * len(stages))(*stages)
+        # whether the fused layers take this network (the limits of islbm_cnn_forward)
+        self.fused = self.lib.islbm_cnn_backward_scratch(
+            len(self.channels), self._chan, base, hidden, 1,
+            ctypes.byref(ctypes.c_ulonglong())) == 0
         self.t = 0
         self.n_params = int(sum(int(np.prod(s)) for n, s in shapes
                                 if not n.startswith("Wc")) +
@@ -113,6 +124,38 @@ class WarmStartNet:
     # ---- forward ----
     def forward(self, z: np.ndarray, keep=True):
         """z: [B, 16] features.  Returns the output [B, S, S, 3] (torch, FP32)."""
+        if not (self.fused and z.shape[1] == FEATURES and 1 <= z.shape[0] <= (1 << 30) // self.size ** 2):
+            return self._forward_chain(z, keep)
+        torch = self.torch
+        B = z.shape[0]
+        z = np.ascontiguousarray(z, dtype=np.float32)
+        shapes, H, stages = [(B, self.base, self.base, self.channels[0])], self.base, len(self.channels)
+        for s, cout in enumerate(self._chan[1:]):
+            H = 2 * H if s + 1 < stages else H
+            shapes.append((B, H, H, cout))
+        # one allocation for everything but the output: features, hidden layer, activations
+        sizes = [B * FEATURES, B * self.hidden] + [math.prod(s) for s in shapes[:-1]]
+        pad = [(n + 63) // 64 * 64 for n in sizes]
+        flat = torch.empty(sum(pad), device=self.device)
+        at, parts = 0, []
+        for n, p in zip(sizes, pad):
+            parts.append(flat[at:at + n])
+            at += p
+        zk, h1 = parts[:2]
+        acts = [a.view(s) for a, s in zip(parts[2:], shapes)]
+        acts.append(torch.empty(shapes[-1], device=self.device))
+        _ck(self.lib.islbm_cnn_forward(stages, self._chan, self.base, self.hidden, self._weights(),
+                                       ctypes.c_void_p(z.ctypes.data), B, _p(zk), _p(h1),
+                                       _ptrs(acts), self._stream()))
+        self.cache = dict(B=B, zk=zk, h1=h1, acts=acts) if keep else None
+        return acts[-1]
+
+    def _weights(self):
+        """The operands of the fused layers, in the order of self.names."""
+        return _ptrs([self.bf.get(n, self.params[n]) for n in self.names])
+
+    def _forward_chain(self, z, keep):
+        """forward() as a chain of im2col GEMMs, for any channel count."""
         torch = self.torch
         B = z.shape[0]
         st = self._stream()
@@ -162,6 +205,18 @@ class WarmStartNet:
         """Gradients of all parameters for the output gradient dy [B, S, S, 3]."""
         torch = self.torch
         c = self.cache
+        if "acts" in c:
+            dy = dy.contiguous()
+            n = ctypes.c_ulonglong()
+            stages = len(self.channels)
+            _ck(self.lib.islbm_cnn_backward_scratch(stages, self._chan, self.base, self.hidden,
+                                                    c["B"], ctypes.byref(n)))
+            scratch = torch.empty(n.value // 4, device=self.device)
+            _ck(self.lib.islbm_cnn_backward(
+                stages, self._chan, self.base, self.hidden, self._weights(), c["B"], _p(c["zk"]),
+                _p(c["h1"]), _ptrs(c["acts"]), _p(dy), _ptrs([self.grads[k] for k in self.names]),
+                _p(scratch), self._stream()))
+            return self.grads
         B = c["B"]
         st = self._stream()
         d = dy.contiguous()
@@ -220,13 +275,13 @@ class WarmStartNet:
 
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.t += 1
-        st = self._stream()
-        for name in self.names:
-            w = self.params[name]
-            _ck(self.lib.islbm_cnn_adam(_p(w), _p(self.bf.get(name)), _p(self.grads[name]),
-                                        _p(self.m[name]), _p(self.v[name]), w.numel(),
-                                        ctypes.c_float(lr), ctypes.c_float(b1), ctypes.c_float(b2),
-                                        ctypes.c_float(eps), self.t, st))
+        names = self.names
+        sizes = (ctypes.c_longlong * len(names))(*[self.params[k].numel() for k in names])
+        _ck(self.lib.islbm_cnn_adam_all(
+            len(names), *[_ptrs([d.get(k) for k in names])
+                          for d in (self.params, self.bf, self.grads, self.m, self.v)],
+            sizes, ctypes.c_float(lr), ctypes.c_float(b1), ctypes.c_float(b2),
+            ctypes.c_float(eps), self.t, self._stream()))
 
     # ---- parameters to / from numpy (checkpoints, oracle comparisons) ----
     def numpy_params(self):

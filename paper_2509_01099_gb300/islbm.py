@@ -43,6 +43,7 @@ EXPORTS = (
     "islbm_cnn_colsum", "islbm_cnn_mse", "islbm_cnn_adam", "islbm_cnn_pack_fields",
     "islbm_cnn_unpack_fields", "islbm_set_row_range", "islbm_get_rows", "islbm_set_rows",
     "islbm_reduce_sums", "islbm_finish_sums", "islbm_cnn_gemm_bf16_ex", "islbm_cnn_check_timeout",
+    "islbm_cnn_forward", "islbm_cnn_backward", "islbm_cnn_backward_scratch", "islbm_cnn_adam_all",
     "islbm_set_allocator",
 )
 REDUCTION_SUMS = 16     # ISLBM_REDUCTION_SUMS of include/islbm.h
@@ -210,6 +211,12 @@ def load_library(build_if_missing: bool = False) -> ctypes.CDLL:
         "islbm_cnn_gemm_bf16": (i, [vp, vp, vp, vp, i, i, i, i, i, i, i, i, i, vp]),
         "islbm_cnn_gemm_bf16_ex": (i, [vp, vp, vp, vp, i, i, i, i, i, i, i, i, i, i, vp]),
         "islbm_cnn_check_timeout": (i, [i, P(i)]),
+        "islbm_cnn_forward": (i, [i, P(i), i, i, P(vp), vp, i, vp, vp, P(vp), vp]),
+        "islbm_cnn_backward_scratch": (i, [i, P(i), i, i, i, P(ctypes.c_ulonglong)]),
+        "islbm_cnn_backward": (i, [i, P(i), i, i, P(vp), i, vp, vp, P(vp), vp, P(vp), vp, vp]),
+        "islbm_cnn_adam_all": (i, [i, P(vp), P(vp), P(vp), P(vp), P(vp), P(ctypes.c_longlong),
+                                   ctypes.c_float, ctypes.c_float, ctypes.c_float,
+                                   ctypes.c_float, ctypes.c_longlong, vp]),
         "islbm_cnn_im2col": (i, [vp, vp, i, i, i, i, i, vp]),
         "islbm_cnn_col2im": (i, [vp, vp, i, i, i, i, i, vp]),
         "islbm_cnn_upsample2x": (i, [vp, vp, i, i, i, i, i, vp]),
