@@ -1488,7 +1488,17 @@ cudaError_t launch_tma(const Solver& s, int cur, S* out, const P2<float>& p) {
 
 dim3 block2() { return dim3(32, 8); }
 dim3 grid2(const Solver& s) { return dim3((s.n[0] + 31) / 32, (s.n[1] + 7) / 8); }
-dim3 grid2_step(const Solver& s) { return dim3((s.n[0] + 31) / 32, (step_rows(s) + 7) / 8); }
+// Rows of a direct step's block (32 columns, one warp a row): 8, fewer where
+// that would leave SMs without a block.  A scheduler's FP64 unit takes 64 cycles
+// for a warp's instruction, so the 243 of a node's FP64 step keep it busy for
+// 7.5 us whatever the mesh: a small mesh has to spread its warps over all SMs
+// (64^2: 16 blocks of 8 warps 18.5 us a step, 128 blocks of one 11.6 us).
+int step_block_rows(const Solver& s) {
+  const long long warps = (long long)((s.n[0] + 31) / 32) * step_rows(s);
+  int rows = 8;
+  while (rows > 1 && warps < 2LL * rows * s.sm_count) rows /= 2;
+  return rows;
+}
 
 // Dispatch on the storage type.
 template <template <typename> class Fn, typename... A>
@@ -1532,10 +1542,12 @@ struct StepFn {
           }
         }
       }
+      const int rows = step_block_rows(s);
+      const dim3 block(32, rows), grid((s.n[0] + 31) / 32, (step_rows(s) + rows - 1) / rows);
       if (s.uniform)
-        k_step<S, true><<<grid2_step(s), block2(), 0, s.stream>>>(in, out, p);
+        k_step<S, true><<<grid, block, 0, s.stream>>>(in, out, p);
       else
-        k_step<S, false><<<grid2_step(s), block2(), 0, s.stream>>>(in, out, p);
+        k_step<S, false><<<grid, block, 0, s.stream>>>(in, out, p);
       return cudaGetLastError();
     }
   }
