@@ -219,6 +219,15 @@ std::string encode_tensor_maps(Solver* s) {
         return "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
     } else {
       std::memcpy(s->tmap_m[b], s->tmap[b], sizeof(s->tmap_m[b]));
+      unsigned yb[3];
+      step_2d_ym_box((int)s->elem, yb);
+      const cuuint32_t ybox[3] = {yb[0], yb[1], yb[2]};
+      r = reinterpret_cast<EncodeFn>(fn)(
+          reinterpret_cast<CUtensorMap*>(s->tmap_y[b]), dt, 3, s->buf[b], dims, strides, ybox, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS)
+        return "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
     }
   }
   return "";
@@ -568,6 +577,11 @@ extern "C" islbm_status islbm_create(const double* xi_x, int nx, const double* x
   s->elem = precision == ISLBM_FP64 ? 8 : (precision == ISLBM_FP32 ? 4 : 2);
   s->pitch = (s->n[0] + 31) / 32 * 32;
   s->plane = (long long)s->pitch * s->n[1] * s->n[2];
+  // two steps a launch where the library chose the kernel (a variant that the
+  // caller named runs as named)
+  s->marching = dim == 2 && prm.kernel == KV_AUTO && s->variant >= KV_TMA_R4S2 &&
+                precision != ISLBM_FP16NEQ &&
+                step_2d_ym_takes(s->n[0], s->n[1], (int)s->elem, (size_t)s->plane * s->elem);
   // FP16NEQ: 14 planes of FP16 remainders, then 4 planes of FP32 moments
   s->state_bytes = precision == ISLBM_FP16NEQ
                        ? (size_t)s->plane * (14 * 2 + 4 * 4)
@@ -826,7 +840,8 @@ static cudaError_t build_graph(Solver* s, int parity) {
   if (e == cudaSuccess) {
     // each captured step gets its own step index (it seeds the stochastic
     // rounding of 16-bit stores; replays repeat the 64 indices)
-    for (int k = 0; k < kGraphSteps && le == cudaSuccess; ++k, ++s->time) le = launch_step(*s);
+    for (int k = 0, done = 0; k < kGraphSteps && le == cudaSuccess; k += done, s->time += done)
+      le = launch_steps(*s, kGraphSteps - k, &done);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(s->side, &g);
     if (e == cudaSuccess && le == cudaSuccess) e = cudaGraphInstantiate(&s->graph[parity], g, 0);
@@ -864,9 +879,11 @@ extern "C" islbm_status islbm_step(islbm_t s, long long n) {
     n -= kGraphSteps;
     s->time += kGraphSteps;
   }
-  for (long long k = 0; k < n; ++k) {
-    CK(s, launch_step(*s));
-    ++s->time;
+  while (n > 0) {
+    int done = 0;
+    CK(s, launch_steps(*s, n, &done));
+    n -= done;
+    s->time += done;
   }
   return ISLBM_OK;
 }
@@ -1126,10 +1143,11 @@ extern "C" islbm_status islbm_load(islbm_t s, const char* path) {
 
 extern "C" islbm_status islbm_debug_bounds(int reset, int* flagged) {
   if (!flagged) return fail(nullptr, ISLBM_ERR_ARG, "islbm_debug_bounds: NULL argument");
-  const int a = bounds_flag_d2(reset), b = bounds_flag_d3(reset), c = bounds_flag_zm(reset);
-  if (a < 0 || b < 0 || c < 0)
+  const int a = bounds_flag_d2(reset), b = bounds_flag_d3(reset);
+  const int c = bounds_flag_zm(reset), d = bounds_flag_ym(reset);
+  if (a < 0 || b < 0 || c < 0 || d < 0)
     return fail(nullptr, ISLBM_ERR_CUDA, "islbm_debug_bounds: reading the flags");
-  *flagged = (a | b | c) ? 1 : 0;
+  *flagged = (a | b | c | d) ? 1 : 0;
   return ISLBM_OK;
 }
 

@@ -1,0 +1,537 @@
+// Marching 2-D step kernel: several time steps in one pass over the state
+// (Sec. 2.1 - 2.3; FP32 and 16-bit deviation storage, node-centred stencil).
+//
+// A CTA owns a strip of up to 64 - 2 (NS - 1) columns over a chunk of rows and
+// marches through it two rows at a time.  NS groups of two warps work as a
+// pipeline: group s computes time step s of the rows that group s - 1 has just
+// finished (group 1 reads rows brought by TMA) and hands its rows on through a
+// ring in shared memory; only the last group writes to global memory.  A thread
+// keeps one column for the whole chunk.
+//
+// Why.  The tile kernel (k_step_tma) moves the whole state through HBM once a
+// step and needs 324 instructions a node, many of them twice: it interpolates
+// 10 rows in x for 8 rows of results, and recomputes tables, flags and
+// addresses for every tile.  Marching interpolates every row once (the rows of
+// the y stencil stay in registers), two rows at a time with the paired FP32
+// instructions, and sets up a column once; with NS = 2 the state crosses HBM
+// once for two steps.
+//
+// Rows.  A group takes the rows of its source in pairs (R, R + 1) and then
+// produces rows (R - 1, R), whose y stencils R - 2 .. R + 1 it has.  The row
+// pairs of consecutive groups are therefore one row apart; a chunk that starts
+// above the bottom wall has group s start 2 (NS - s) rows below it.  The clamped
+// stencils at the walls (row 0: rows 0 .. 2; row n - 1: rows n - 3 .. n - 1)
+// fit the window when row 0 is the first and row n - 1 the second of a produced
+// pair: chunks that touch the top wall have an even number of rows.
+//
+// The operations and their order are those of tile_body, and intermediate rows
+// are rounded to the storage type as a store would (stochastic rounding
+// included), so the results are the same bits as single steps.
+//
+// Every wait is bounded; a wait that gives up raises the CTA's abort flag and
+// the error flag, thread 0 waits for its copies in flight, and the CTA returns.
+#include <algorithm>
+#include <type_traits>
+
+#include "islbm_d2_common.cuh"
+#include "islbm_store.cuh"
+#include "islbm_tma.cuh"
+
+namespace islbm {
+namespace {
+
+constexpr int kYmW = 64;           // columns of a group
+constexpr int kYmMinRows = 12;     // shortest chunk
+
+template <typename S, int NS>
+struct YmGeom {
+  static constexpr int HX = 16 / (int)sizeof(S);       // elements of a 16-byte chunk
+  // staged row: the columns of group 1 with one halo column on each side, from
+  // a 16-byte boundary
+  static constexpr int TW = (kYmW + 2 + HX - 1 + HX - 1) / HX * HX;
+  // row pitch of the rings between groups, whose rows are FP32 in every storage
+  // form (rounded to it, so that the next group reads them without conversions)
+  static constexpr int RW = kYmW + 2;
+  static constexpr unsigned TMA_BYTES = 14u * 2u * TW * sizeof(S);
+  static constexpr unsigned RING_BYTES = (14u * 2u * RW * 4u + 127u) / 128u * 128u;
+  static constexpr int DT = 3;                         // TMA stages (row pairs)
+  static constexpr int DR = 4;                         // row pairs of a ring
+  static constexpr unsigned SMEM = DT * TMA_BYTES + (NS - 1) * DR * RING_BYTES + 256;
+  static constexpr int THREADS = NS * 64;
+  static_assert(TMA_BYTES % 128 == 0, "stages keep the TMA's 128-byte alignment");
+  static_assert((2 * DT + 2 * DR * (NS - 1)) * 8 + 4 <= 256 - 16, "barriers and the flag");
+};
+
+// The items of a launch: strips of columns x chunks of rows, evenly split.
+struct YmSched {
+  int nstrip, nchunk;
+  __host__ __device__ int row(int k, int n) const {   // first row of chunk k
+    if (k >= nchunk) return n;
+    const int r = (int)((long long)n * k / nchunk);
+    return k > 0 && k == nchunk - 1 ? r - ((n - r) & 1) : r;   // the top chunk is even
+  }
+  __host__ __device__ int col(int k, int n) const { return (int)((long long)n * k / nstrip); }
+};
+
+// y tables of two rows, cy = +1 and -1.
+struct YmTables {
+  float4 p0, p1, m0, m1;
+};
+
+// Wait on `bar`; one that does not end in time raises the error flag and the
+// CTA's abort flag, with which every later wait returns at once: the groups
+// run to their ends without waiting (their results are void).
+__device__ __noinline__ void ym_wait_slow(uint64_t* bar, unsigned phase, volatile int* abort,
+                                          int* err) {
+  if (*abort) return;
+  if (!mbar_wait_or_abort(bar, phase, abort)) {
+    if (!*abort) atomicExch(err, 1);
+    *abort = 1;
+  }
+}
+__device__ __forceinline__ void ym_wait(uint64_t* bar, unsigned phase, volatile int* abort,
+                                        int* err) {
+  if (!mbar_try_wait(bar, phase)) ym_wait_slow(bar, phase, abort, err);
+}
+
+// Group of step s (1 .. NS) of one item.  SRC: element type of the source rows
+// (plane pitch PS, row pitch RS).  First rows are at `src_ring`.
+template <typename S, int NS, int s>
+struct YmGroup {
+  using G = YmGeom<S, NS>;
+  static constexpr bool FIRST = s == 1, LAST = s == NS;
+  using T = std::conditional_t<FIRST, S, float>;       // type of the source rows
+  static constexpr int RS = FIRST ? G::TW : G::RW;     // row pitch of the source
+  static constexpr int PS = 2 * RS;                    // plane pitch of the source
+
+  // per-thread state of the march
+  float2 hp[8];       // previous row pair of the planes moving in y (x-interpolated)
+  float sv[6];        // second row of the previous pair, the planes not moving in y
+  float bb[2];        // raw planes 7, 8 of row 0
+  float2 wp[3], wm[3];
+  int ci, bp, bm;     // source columns: own, stencil bases of cx = +1, -1
+  bool wW, wE, any;
+
+  static __device__ __forceinline__ float2 own(const T* a, const T* b, int pl, int c) {
+    return make_float2(to_f(a[pl * PS + c]), to_f(b[pl * PS + c]));
+  }
+  static __device__ __forceinline__ float2 interp(const T* a, const T* b, int pl, int c,
+                                                  const float2 (&w)[3]) {
+    return __ffma2_rn(w[2], own(a, b, pl, c + 2),
+                      __ffma2_rn(w[1], own(a, b, pl, c + 1), __fmul2_rn(w[0], own(a, b, pl, c))));
+  }
+
+  __device__ __forceinline__ void setup(const P2<float>& p, int x, int src0) {
+    const int xc = min(max(x, 0), p.nx - 1);
+    const float4 a = __ldg(p.px[0] + xc), b = __ldg(p.px[1] + xc);
+    wp[0] = make_float2(a.x, a.x);
+    wp[1] = make_float2(a.y, a.y);
+    wp[2] = make_float2(a.z, a.z);
+    wm[0] = make_float2(b.x, b.x);
+    wm[1] = make_float2(b.y, b.y);
+    wm[2] = make_float2(b.z, b.z);
+    ci = x - src0;
+    bp = __float_as_int(a.w) - src0;
+    bm = __float_as_int(b.w) - src0;
+    if (!(ISLBM_IN_WINDOW(ci, RS) && ISLBM_IN_WINDOW(bp, RS) && ISLBM_IN_WINDOW(bm, RS)))
+      ci = bp = bm = 0;
+    wW = x == 0;
+    wE = x == p.nx - 1;
+    any = __any_sync(0xffffffffu, wW || wE);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) hp[k] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sv[k] = 0.f;
+    bb[0] = bb[1] = 0.f;
+  }
+
+  // Takes source rows R (at a) and R + 1 (at b), produces rows R - 1 and R into
+  // fn, gn (of the first call: nothing of use).  One copy of this code serves
+  // every iteration, the walls' behind uniform branches: the groups run
+  // different code at the same time, and with separate copies for the first
+  // and last rows (and the loop unrolled) instruction fetch made the kernel
+  // slower by a fifth.
+  __device__ __forceinline__ void take(const P2<float>& p, const T* a, const T* b, int R,
+                                       const YmTables& q, float2 (&fn)[9], float2 (&gn)[5]) {
+    const bool bot = R == 1, top = R == p.ny - 1, edge = bot || top;
+    // y pass of window slot k: rows R - 2, R - 1 (hp) and R, R + 1 (h)
+    auto ypass = [&](int k, float2 h, bool plus, float2& out) {
+      const float4 q0 = plus ? q.p0 : q.m0, q1 = plus ? q.p1 : q.m1;
+      out.x = dot3(q0, hp[k].x, hp[k].y, h.x);
+      out.y = dot3(q1, hp[k].y, h.x, h.y);
+      if (edge) {
+        if (bot && !plus) out.x = dot3(q0, hp[k].y, h.x, h.y);
+        if (top && plus) out.y = dot3(q1, hp[k].x, hp[k].y, h.x);
+      }
+    };
+    // planes that do not move in y
+    auto still = [&](int k, float2 z, float2& out) {
+      out = make_float2(sv[k], z.x);
+      sv[k] = z.y;
+    };
+    still(0, own(a, b, 0, ci), fn[0]);
+    still(1, own(a, b, 9, ci), gn[0]);
+    float2 z1 = interp(a, b, 1, bp, wp), z3 = interp(a, b, 3, bm, wm);
+    float2 t1 = interp(a, b, 10, bp, wp), t3 = interp(a, b, 12, bm, wm);
+    if (any) {
+      if (wW) {
+        z1 = own(a, b, 3, ci);
+        const float2 v = own(a, b, 12, ci);
+        t1 = make_float2(p.abb_hot - v.x, p.abb_hot - v.y);
+      }
+      if (wE) {
+        z3 = own(a, b, 1, ci);
+        const float2 v = own(a, b, 10, ci);
+        t3 = make_float2(p.abb_cold - v.x, p.abb_cold - v.y);
+      }
+    }
+    still(2, z1, fn[1]);
+    still(3, z3, fn[3]);
+    still(4, t1, gn[1]);
+    still(5, t3, gn[3]);
+    // planes moving in y only
+    auto straight = [&](int kp, int plp, int km, int plm, float2& outp, float2& outm) {
+      const float2 h = own(a, b, plp, ci), g = own(a, b, plm, ci);
+      ypass(kp, h, true, outp);
+      ypass(km, g, false, outm);
+      if (edge) {
+        if (bot) outp.x = hp[km].y;
+        if (top) outm.y = h.x;
+      }
+      hp[kp] = h;
+      hp[km] = g;
+    };
+    straight(0, 2, 1, 4, fn[2], fn[4]);
+    straight(2, 11, 3, 13, gn[2], gn[4]);
+    // diagonals.  Next to an x-wall the window holds the raw bounce-back
+    // partner instead of the interpolated plane, and its centre is the result.
+    auto diag = [&](int k, int pl, int partner, bool plus_x, bool plus_y, float2& out) {
+      float2 h = plus_x ? interp(a, b, pl, bp, wp) : interp(a, b, pl, bm, wm);
+      ypass(k, h, plus_y, out);
+      if (any) {
+        if (plus_x ? wW : wE) {
+          h = own(a, b, partner, ci);
+          out = make_float2(hp[k].y, h.x);
+        }
+      }
+      hp[k] = h;
+    };
+    diag(4, 5, 7, true, true, fn[5]);
+    diag(5, 6, 8, false, true, fn[6]);
+    diag(6, 7, 5, false, false, fn[7]);
+    diag(7, 8, 6, true, false, fn[8]);
+    if (edge) {
+      if (bot) {
+        fn[5].x = bb[0];
+        fn[6].x = bb[1];
+      }
+      if (top) {
+        fn[7].y = to_f(a[5 * PS + ci]);
+        fn[8].y = to_f(a[6 * PS + ci]);
+      }
+    }
+    if (R < 0) {
+      bb[0] = to_f(b[7 * PS + ci]);
+      bb[1] = to_f(b[8 * PS + ci]);
+    }
+  }
+};
+
+template <typename S, int NS, int MINB>
+__global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
+    k_step_ym(const __grid_constant__ CUtensorMap tmap, S* __restrict__ fout, P2<float> p,
+              const __grid_constant__ PairC kc, int* err, YmSched sc) {
+  using G = YmGeom<S, NS>;
+  constexpr int DT = G::DT, DR = G::DR;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* rings = smem_raw + DT * G::TMA_BYTES;
+  // full / empty barriers of the TMA stages, then of each ring
+  uint64_t* bars = reinterpret_cast<uint64_t*>(rings + (NS - 1) * DR * G::RING_BYTES + 16);
+  volatile int* abort = reinterpret_cast<volatile int*>(bars + 2 * DT + 2 * DR * (NS - 1));
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < DT; ++k) {
+      mbar_init(&bars[k], 1);
+      mbar_init(&bars[DT + k], 2);
+    }
+    for (int k = 0; k < 2 * DR * (NS - 1); ++k) mbar_init(&bars[2 * DT + k], 2);
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+
+  const int strip = blockIdx.x % sc.nstrip, chunk = blockIdx.x / sc.nstrip;
+  const int x0 = sc.col(strip, p.nx), x1 = sc.col(strip + 1, p.nx);
+  const int ya = sc.row(chunk, p.ny), yb = sc.row(chunk + 1, p.ny);
+  const int nI = (yb - ya + 1) / 2;           // row pairs of the last group
+  const bool at_bottom = ya == 0, at_top = yb == p.ny;
+  // group s: iterations [first(s), last(s)], rows ya - 2 (NS - s) - 1 + 2 i, +1
+  auto first = [&](int s) { return at_bottom ? NS - s : 0; };
+  auto last = [&](int s) { return nI + (at_top ? NS - s : 2 * (NS - s)); };
+  const int xa = (x0 - NS) & ~(G::HX - 1);    // first staged column
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // Copies of group 1's iterations, by thread 0: one box of a row pair, all planes.
+  const int copies = last(1) - first(1) + 1, row0 = ya - 2 * (NS - 1) - 1 + 2 * first(1);
+  int issued = 0;
+  auto issue = [&]() {
+    const int st = issued % DT;
+    mbar_expect_tx(&bars[st], G::TMA_BYTES);
+    tma_load_3d(smem_raw + st * G::TMA_BYTES, &tmap, xa, row0 + 2 * issued, 0, &bars[st]);
+    ++issued;
+  };
+  if (threadIdx.x == 0) {
+    asm volatile("prefetch.tensormap [%0];\n" ::"l"(&tmap) : "memory");
+    grid_launch_next();
+    grid_wait();
+    while (issued < min(DT, copies)) issue();
+  }
+  auto run = [&](auto step) {
+    constexpr int s = decltype(step)::value;
+    using Gr = YmGroup<S, NS, s>;
+    using T = typename Gr::T;
+    constexpr bool FIRST = Gr::FIRST, LAST = Gr::LAST;
+    const int c = threadIdx.x - 64 * (s - 1);
+    const int x = x0 - (NS - s) + c;
+    const int src0 = FIRST ? xa : x0 - NS + s - 1;
+    Gr g;
+    g.setup(p, x, src0);
+    // source: the TMA stages or ring s - 2 (between groups s - 1 and s); target: ring s - 1
+    uint64_t* sfull = FIRST ? bars : bars + 2 * DT + 2 * DR * (s - 2);
+    uint64_t* sempty = sfull + (FIRST ? DT : DR);
+    uint64_t* tfull = bars + 2 * DT + 2 * DR * (s - 1);
+    uint64_t* tempty = tfull + DR;
+    constexpr int DS = FIRST ? DT : DR;
+    const unsigned char* src = FIRST ? smem_raw : rings + (s - 2) * DR * G::RING_BYTES;
+    constexpr unsigned SB = FIRST ? G::TMA_BYTES : G::RING_BYTES;
+    unsigned char* target = rings + (s - 1) * DR * G::RING_BYTES;
+    const int i0 = first(s), i1 = last(s);
+    const bool mine = x >= x0 && x < x1;
+    int ss = 0;              // source slot of this iteration's (first) row pair
+    unsigned sp = 0;         // its phase
+    int ts = 0;              // target slot
+    unsigned tp = 1;         // phase of its empty barrier (1: the first use passes)
+    // source rows of iteration i: FIRST: both of stage ss; else the second row of
+    // pair i (slot ss) and the first row of pair i + 1 (the next slot)
+    if (!FIRST && !at_bottom) ym_wait(&sfull[0], 0u, abort, err);
+    // a bottom chunk has no pair i0: its first pair is taken as "next"
+    int have = FIRST || !at_bottom ? 1 : 0;
+    unsigned off = 0;        // byte offset of the last group's next output row
+    if (LAST) off = (unsigned)(((size_t)ya * p.pitch + (mine ? x : x0)) * sizeof(S));
+    const int first_row = ya - 2 * (NS - s) + 2 * i0;
+    const float4 *tqp = p.py[0] + first_row, *tqm = p.py[1] + first_row;
+    for (int i = i0; i <= i1; ++i) {
+      const int R = ya - 2 * (NS - s) - 1 + 2 * i;
+      // tables of rows R - 1 and R, loaded before the wait, which hides their latency
+      YmTables q{};
+      if (i > i0) {
+        q = YmTables{__ldg(tqp), __ldg(tqp + 1), __ldg(tqm), __ldg(tqm + 1)};
+        tqp += 2;
+        tqm += 2;
+      }
+      const T *a, *b;
+      int ns = ss;
+      unsigned np = sp;
+      if (FIRST) {
+        ym_wait(&sfull[ss], sp, abort, err);
+        a = reinterpret_cast<const T*>(src + ss * SB);
+        b = a + Gr::RS;
+      } else {
+        if (have && ++ns == DS) {
+          ns = 0;
+          np ^= 1u;
+        }
+        // the pair after the last one of a chunk at the top wall does not exist
+        // (row ny, which no result uses)
+        if (!(at_top && i == i1)) ym_wait(&sfull[ns], np, abort, err);
+        a = reinterpret_cast<const T*>(src + ss * SB) + Gr::RS;
+        b = reinterpret_cast<const T*>(src + ns * SB);
+      }
+      float2 fn[9], gn[5];
+      g.take(p, a, b, R, q, fn, gn);
+      // the source rows are in registers: release stage / pair i
+      __syncwarp();
+      if (have && lane == 0) mbar_arrive(&sempty[ss]);
+      if (FIRST && threadIdx.x == 0 && i > i0 && issued < copies) {
+        // refill the stage of the iteration before, which the other warp has
+        // released by now (or does within this iteration)
+        const int n = issued - DT;
+        ym_wait(&sempty[n % DT], (unsigned)(n / DT) & 1u, abort, err);
+        if (!*abort) {
+          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+          issue();
+        }
+      }
+      if (FIRST) {
+        if (++ss == DS) {
+          ss = 0;
+          sp ^= 1u;
+        }
+      } else {
+        ss = ns;
+        sp = np;
+        have = 1;
+      }
+      if (i == i0) continue;
+      float2 mm[4];
+      collide_pair(fn, gn, kc, mm);
+      auto val = [&](int k) { return k < 9 ? fn[k < 9 ? k : 0] : gn[k < 9 ? 0 : k - 9]; };
+      const unsigned seed_step = p.step + (unsigned)(s - 1);
+      if constexpr (LAST) {
+        if (mine) {
+          char* o = reinterpret_cast<char*>(fout);
+          const size_t ps = (size_t)p.plane * sizeof(S);
+          unsigned r = sr_seed((size_t)(R - 1) * p.pitch + x, seed_step);
+#pragma unroll
+          for (int k = 0; k < 14; ++k)
+            Store<S>::st_sr(reinterpret_cast<S*>(o + k * ps + off), val(k).x, sr_next(r));
+          if (R < yb) {
+            const unsigned off1 = off + (unsigned)(p.pitch * sizeof(S));
+            unsigned r1 = sr_seed((size_t)R * p.pitch + x, seed_step);
+#pragma unroll
+            for (int k = 0; k < 14; ++k)
+              Store<S>::st_sr(reinterpret_cast<S*>(o + k * ps + off1), val(k).y, sr_next(r1));
+          }
+        }
+        off += (unsigned)(2 * p.pitch * sizeof(S));
+      } else {
+        ym_wait(&tempty[ts], tp, abort, err);
+        float* t = reinterpret_cast<float*>(target + ts * G::RING_BYTES) + c;
+        unsigned r = sr_seed((size_t)((long long)(R - 1) * p.pitch + x), seed_step);
+        unsigned r1 = sr_seed((size_t)((long long)R * p.pitch + x), seed_step);
+#pragma unroll
+        for (int k = 0; k < 14; ++k) {
+          t[k * 2 * G::RW] = Store<S>::rounded_sr(val(k).x, sr_next(r));
+          t[k * 2 * G::RW + G::RW] = Store<S>::rounded_sr(val(k).y, sr_next(r1));
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tfull[ts]);
+        if (++ts == DR) {
+          ts = 0;
+          tp ^= 1u;
+        }
+      }
+    }
+  };
+  if (warp < 2)
+    run(std::integral_constant<int, 1>{});
+  else if constexpr (NS > 1)
+    run(std::integral_constant<int, 2>{});
+  // copies still in flight land before the CTA's shared memory is released
+  if (threadIdx.x == 0)
+    for (int k = max(0, issued - DT); k < issued; ++k)
+      mbar_wait(&bars[k % DT], (unsigned)(k / DT) & 1u);
+}
+
+// Strips and chunks of a launch.  A CTA costs its rows and about kYmStart more
+// (the rows below its chunk that the first groups compute, the pipeline's fill
+// and drain).  kYmRow: relative time of a row with 1 .. 4 CTAs on an SM; the
+// warps of few CTAs leave issue slots empty, so four CTAs take only 1.7 times
+// as long as one (measured at 257^2 .. 4096^2 with 5 .. 71 chunks; 1024^2: 26
+// chunks, three CTAs an SM, 16.6 us a step, 35 chunks, four, 15.9).
+constexpr double kYmStart = 8.0;
+constexpr double kYmRow[5] = {0.0, 0.25, 0.30, 0.345, 0.42};
+
+template <int NS>
+YmSched ym_schedule(int nx, int ny, int sms, int per_sm) {
+  YmSched sc;
+  const int w = kYmW - 2 * (NS - 1);
+  sc.nstrip = (nx + w - 1) / w;
+  sc.nchunk = 1;
+  double best = 1e300;
+  for (int c = ny % 2 ? 2 : 1; c <= ny / kYmMinRows; ++c) {
+    const long long items = (long long)sc.nstrip * c;
+    const long long slots = (long long)sms * per_sm, left = items % slots;
+    const double rows = (double)((ny + c - 1) / c) + kYmStart;
+    const double cost = rows * ((double)(items / slots) * kYmRow[std::min(per_sm, 4)] +
+                                kYmRow[std::min<long long>(4, (left + sms - 1) / sms)]);
+    if (cost < best - 1e-9) {
+      best = cost;
+      sc.nchunk = c;
+    }
+  }
+  return sc;
+}
+
+template <typename S, int NS>
+cudaError_t launch_ym(Solver& s) {
+  using G = YmGeom<S, NS>;
+  constexpr int MINB = NS == 2 ? 4 : 6;
+  const auto k = k_step_ym<S, NS, MINB>;
+  int per_sm = 0;
+  const cudaError_t e = launch_setup_once(
+      reinterpret_cast<const void*>(k),
+      [](const void* f, int* n) {
+        cudaError_t e2 =
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+        if (e2 == cudaSuccess)
+          e2 = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    cudaSharedmemCarveoutMaxShared);
+        if (e2 == cudaSuccess)
+          e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, f, G::THREADS, G::SMEM);
+        return e2;
+      },
+      &per_sm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const YmSched sc = ym_schedule<NS>(s.n[0], s.n[1], s.sm_count, per_sm);
+  const P2<float> p = make_params<float>(s);
+  // a launch that fills the GPU's slots leaves the next one's early blocks only
+  // those that come free; into a half-full GPU they would crowd on the SMs with
+  // room (1024^2, 35 chunks, 595 of 608 slots: 15.9 -> 15.4 us a step; 26 chunks,
+  // 442 slots: 16.6 -> 19.4 us)
+  const bool serial = sc.nstrip * sc.nchunk >= s.sm_count * per_sm * 15 / 16;
+  return launch_grid(serial, k, sc.nstrip * sc.nchunk, G::THREADS, G::SMEM, s.stream,
+                     *reinterpret_cast<const CUtensorMap*>(s.tmap_y[s.cur]),
+                     static_cast<S*>(s.buf[s.cur ^ 1]), p, make_pair_constants(p), s.derr, sc);
+}
+
+}  // namespace
+
+// Whether the marching kernel takes a mesh (at least two chunks of the shortest
+// length, 32-bit offsets in a plane), and whether it is the faster one there: it
+// is once its CTAs fill the GPU, and in the 16-bit forms, which are bound by
+// their conversions and stochastic rounding in either kernel, on larger meshes
+// only.  us a step, tile kernel and this one: FP32 512^2 6.5 / 7.0, 900^2 15.9 /
+// 15.3, 1024^2 19.4 / 15.4, 2049^2 74 / 54, 4096^2 277 / 193; BF16 1024^2 18.2 /
+// 18.4, 1400^2 32.4 / 30.6, 4096^2 246 / 234.
+constexpr long long kYmMinNodes = 600000, kYmMinNodes16 = 1500000;
+bool step_2d_ym_takes(int nx, int ny, int elem, size_t plane_bytes) {
+  return nx >= 16 && ny >= 2 * kYmMinRows + 2 && plane_bytes < (size_t)1 << 31 &&
+         (long long)nx * ny >= (elem == 4 ? kYmMinNodes : kYmMinNodes16);
+}
+
+// TMA box (x, y, planes) of a staged row pair.
+void step_2d_ym_box(int elem, unsigned (&box)[3]) {
+  box[0] = (unsigned)(elem == 4 ? YmGeom<float, 2>::TW : YmGeom<__half, 2>::TW);
+  box[1] = 2;
+  box[2] = 14;
+}
+
+cudaError_t launch_step_2d_ym(Solver& s, int steps) {
+  if (steps != 2) return cudaErrorInvalidValue;
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (s.precision) {
+    case ISLBM_FP32: e = launch_ym<float, 2>(s); break;
+    case ISLBM_FP16DEV: e = launch_ym<__half, 2>(s); break;
+    case ISLBM_BF16DEV: e = launch_ym<__nv_bfloat16, 2>(s); break;
+  }
+  if (e == cudaSuccess) s.cur ^= 1;
+  return e;
+}
+
+int bounds_flag_ym(int reset) {
+#ifdef ISLBM_BOUNDS_CHECK
+  int v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_bounds_flag, sizeof(int)) != cudaSuccess) return -1;
+  if (reset) {
+    const int zero = 0;
+    cudaMemcpyToSymbol(g_bounds_flag, &zero, sizeof(int));
+  }
+  return v;
+#else
+  (void)reset;
+  return 0;
+#endif
+}
+
+}  // namespace islbm

@@ -35,6 +35,7 @@ __device__ __forceinline__ bool in_window(int v, int n) {
 int bounds_flag_d2(int reset);
 int bounds_flag_d3(int reset);
 int bounds_flag_zm(int reset);
+int bounds_flag_ym(int reset);
 
 // Device memory of the library: through the allocator registered with
 // islbm_set_allocator, else cudaMallocAsync / cudaFreeAsync on the stream of
@@ -54,6 +55,36 @@ void dev_free(const DevAllocator& a, void* p, cudaStream_t stream);
 // setup stored (e.g. CTAs per SM).
 cudaError_t launch_setup_once(const void* kernel, cudaError_t (*setup)(const void*, int*),
                               int* value);
+
+// Programmatic serialisation of step kernels (serial = true): the next step's
+// blocks may start, set up their barriers and tables (which no kernel writes)
+// and wait (grid_wait) as soon as every block of this one has started
+// (grid_launch_next).  grid_wait returns once the grids before are complete and
+// their writes visible; a block touches the state only after it.  Both are
+// no-ops in an ordinary launch.
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+__device__ __forceinline__ void grid_launch_next() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_grid(bool serial, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                        cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = serial ? 1 : 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
 
 // NVTX range for profilers (nsys / ncu ranges); a no-op when no tool is attached.
 struct NvtxRange {
@@ -172,6 +203,8 @@ struct Solver {
   int* derr = nullptr;
   alignas(128) unsigned char tmap[2][128];   // TMA descriptors of buf[0] / buf[1]
   alignas(128) unsigned char tmap_m[2][128]; // FP16NEQ: of their moment planes
+  alignas(128) unsigned char tmap_y[2][128]; // of a row pair (the 2-D marching kernel)
+  bool marching = false;          // 2-D: two steps in one launch where two are due
   alignas(128) unsigned char tmap3[2][7][128];   // 3-D: one descriptor per box shape
   // CUDA graphs of kGraphSteps steps, one per starting buffer, replayed on a
   // private stream that is ordered against `stream` with events
@@ -201,6 +234,13 @@ cudaError_t launch_populations(Solver& s, double* f, double* g);
 // Reductions of the current state into s.hresult: RED_COUNT sums and, at
 // RED_STRIDE, the step kernels' error flag (valid once the stream is idle).
 cudaError_t launch_reduce(Solver& s);
+
+// Up to `want` >= 1 steps in one launch; *done receives how many.
+cudaError_t launch_steps(Solver& s, long long want, int* done);
+// 2-D marching kernel (two steps a launch): whether it takes a mesh, its TMA box
+cudaError_t launch_step_2d_ym(Solver& s, int steps);
+bool step_2d_ym_takes(int nx, int ny, int elem, size_t plane_bytes);
+void step_2d_ym_box(int elem, unsigned (&box)[3]);
 
 cudaError_t launch_init_fields_3d(Solver& s, const double* rho, const double* T,
                                   const double* u0, const double* u1, const double* u2);

@@ -30,6 +30,8 @@ struct Store<float> {
   static __device__ __forceinline__ R ld(const float* p) { return __ldg(p); }
   static __device__ __forceinline__ void st(float* p, R v) { *p = v; }
   static __device__ __forceinline__ void st_sr(float* p, R v, unsigned) { *p = v; }
+  // the value that st_sr would leave in the storage, as the compute type reads it
+  static __device__ __forceinline__ R rounded_sr(R v, unsigned) { return v; }
 };
 
 // Stochastic rounding of the 16-bit stores of the time step.  Near a steady
@@ -57,6 +59,9 @@ struct Store<__half> {
   static __device__ __forceinline__ void st_sr(__half* p, R v, unsigned r) {
     *p = sr_to_fp16(v, r);
   }
+  static __device__ __forceinline__ R rounded_sr(R v, unsigned r) {
+    return __half2float(sr_to_fp16(v, r));
+  }
 };
 
 template <>
@@ -73,6 +78,9 @@ struct Store<__nv_bfloat16> {
     // half (the carry rounds away from zero with the dropped fraction's
     // probability) and keep the upper half
     *p = __ushort_as_bfloat16((unsigned short)((__float_as_uint(v) + (r >> 16)) >> 16));
+  }
+  static __device__ __forceinline__ R rounded_sr(R v, unsigned r) {
+    return __uint_as_float((__float_as_uint(v) + (r >> 16)) & 0xFFFF0000u);
   }
 };
 
