@@ -988,7 +988,9 @@ __global__ void __launch_bounds__(kThreads, (tma_ctas_per_sm<S, R, STAGES>()))
     __syncthreads();
     int filled = 0;   // thread 0: stage uses filled so far (copies or a plain arrival)
     int seen = 0;     // thread 0: stage uses whose phase it has seen complete
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
+      grid_launch_next();
+      grid_wait();
       for (int st = 0; st < STAGES; ++st) {
         const int t = blockIdx.x + st * gridDim.x;
         if (t < ntiles) {
@@ -996,6 +998,7 @@ __global__ void __launch_bounds__(kThreads, (tma_ctas_per_sm<S, R, STAGES>()))
           filled = st + 1;
         }
       }
+    }
     const unsigned lane = threadIdx.x & 31u;
     auto fail = [&]() {
       if (!*abort) atomicExch(&sched[0], 1);
@@ -1301,10 +1304,14 @@ cudaError_t launch_tma(const Solver& s, int cur, S* out, const P2<float>& p) {
   const int grid = std::min(ntiles, s.sm_count * blocks_per_sm);
   // claimed tiles pay off once a CTA walks more than a few dozen tiles
   const int k0 = tma_first_claim(ntiles, grid, STAGES);
-  k_step_tma<S, R, STAGES><<<grid, kThreads, smem, s.stream>>>(
-      *reinterpret_cast<const CUtensorMap*>(s.tmap[cur]),
-      *reinterpret_cast<const CUtensorMap*>(s.tmap_m[cur]), out, p, s.derr, k0);
-  return cudaGetLastError();
+  // few tiles a CTA: the launch gap is a good part of the step (FP32 64 x 8
+  // tiles, 257^2 4.5 -> 4.2 us, 512^2 7.0 -> 6.5); beyond, and in the 64 x 16
+  // tiles of the 16-bit forms, early blocks cost more than they hide (BF16
+  // 1024^2 18.3 -> 21.2 us)
+  const bool serial = std::is_same<S, float>::value && R == 2 && ntiles <= 4 * grid;
+  return launch_grid(serial, k_step_tma<S, R, STAGES>, grid, kThreads, smem, s.stream,
+                     *reinterpret_cast<const CUtensorMap*>(s.tmap[cur]),
+                     *reinterpret_cast<const CUtensorMap*>(s.tmap_m[cur]), out, p, s.derr, k0);
 }
 
 dim3 block2() { return dim3(32, 8); }
