@@ -165,6 +165,149 @@ __global__ void __launch_bounds__(256)
   for (int i = 0; i < 5; ++i) St::st_sr(fout + (9 + i) * P + idx, g[i], sr_next(r));
 }
 
+// The FP64 step of a small mesh: four warps share the 32 nodes of a block.
+// A scheduler's FP64 unit takes 64 cycles for a warp's instruction, and a warp
+// alone on its SM has the other three units idle: k_step spends 243 of them in
+// a row (7.5 us).  Here each warp pulls a quarter of the populations, then
+// computes a part of the moments, of their relaxation and of the outputs,
+// handed on through shared memory: about 75 instructions a warp.  64^2: 11.6 ->
+// 5.1 us a step.
+template <bool UNI>
+__global__ void __launch_bounds__(128)
+    k_step_split(const double* __restrict__ fin, double* __restrict__ fout, P2<double> p) {
+  using St = Store<double>;
+  __shared__ double sf[14][32];   // pulled populations
+  __shared__ double sm[16][32];   // shared intermediate results
+  enum { DRHO, INV, JX, JY, TR, A1, A2, A4, A5, A6, A7, A8 };
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int xt = blockIdx.x * 32 + lane, x = min(xt, p.nx - 1), y = p.y0 + (int)blockIdx.y;
+  const size_t idx = (size_t)y * p.pitch + x;
+  const long long P = p.plane;
+  const bool wW = (x == 0), wE = (x == p.nx - 1), wS = (y == 0), wN = (y == p.ny - 1);
+  const double* gin = fin + 9 * P;
+  auto f_at = [&](int i) { return St::ld(fin + i * P + idx); };
+  auto g_at = [&](int i) { return St::ld(gin + i * P + idx); };
+  // walls as in k_step
+  if (warp == 0) {
+    const double a = wW ? f_at(3) : pull<double, double, 1, 0, UNI>(fin + P, x, y, p);
+    const double b = (wW || wS) ? f_at(7) : pull<double, double, 1, 1, UNI>(fin + 5 * P, x, y, p);
+    const double c = wW ? p.abb_hot - g_at(3) : pull<double, double, 1, 0, UNI>(gin + P, x, y, p);
+    sf[0][lane] = f_at(0);
+    sf[1][lane] = a;
+    sf[5][lane] = b;
+    sf[10][lane] = c;
+  } else if (warp == 1) {
+    const double a = wS ? f_at(4) : pull<double, double, 0, 1, UNI>(fin + 2 * P, x, y, p);
+    const double b = (wE || wS) ? f_at(8) : pull<double, double, -1, 1, UNI>(fin + 6 * P, x, y, p);
+    const double c = wS ? g_at(4) : pull<double, double, 0, 1, UNI>(gin + 2 * P, x, y, p);
+    sf[9][lane] = g_at(0);
+    sf[2][lane] = a;
+    sf[6][lane] = b;
+    sf[11][lane] = c;
+  } else if (warp == 2) {
+    const double a = wE ? f_at(1) : pull<double, double, -1, 0, UNI>(fin + 3 * P, x, y, p);
+    const double b = (wE || wN) ? f_at(5) : pull<double, double, -1, -1, UNI>(fin + 7 * P, x, y, p);
+    const double c =
+        wE ? p.abb_cold - g_at(1) : pull<double, double, -1, 0, UNI>(gin + 3 * P, x, y, p);
+    sf[3][lane] = a;
+    sf[7][lane] = b;
+    sf[12][lane] = c;
+  } else {
+    const double a = wN ? f_at(2) : pull<double, double, 0, -1, UNI>(fin + 4 * P, x, y, p);
+    const double b = (wW || wN) ? f_at(6) : pull<double, double, 1, -1, UNI>(fin + 8 * P, x, y, p);
+    const double c = wN ? g_at(2) : pull<double, double, 0, -1, UNI>(gin + 4 * P, x, y, p);
+    sf[4][lane] = a;
+    sf[8][lane] = b;
+    sf[13][lane] = c;
+  }
+  __syncthreads();
+  auto f = [&](int i) { return sf[i][lane]; };
+  auto g = [&](int i) { return sf[9 + i][lane]; };
+  // the sums of collide_m
+  if (warp == 0) {
+    const double drho = ((f(0) + f(1)) + (f(2) + f(3))) + ((f(4) + f(5)) + (f(6) + f(7))) + f(8);
+    sm[DRHO][lane] = drho;
+    sm[INV][lane] = 1.0 / (1.0 + drho);
+  } else if (warp == 1) {
+    sm[JX][lane] = (f(1) - f(3)) + (f(5) - f(6)) + (f(8) - f(7));
+  } else if (warp == 2) {
+    sm[JY][lane] = (f(2) - f(4)) + (f(5) + f(6)) - (f(7) + f(8));
+  } else {
+    sm[TR][lane] = ((g(0) + g(1)) + (g(2) + g(3))) + g(4);
+  }
+  __syncthreads();
+  const double drho = sm[DRHO][lane], rho = 1.0 + drho, inv = sm[INV][lane], Tr = sm[TR][lane];
+  const double Fy = rho * p.gbeta * (Tr + p.Fb);
+  const double ux = sm[JX][lane] * inv, uy = fma(0.5, Fy, sm[JY][lane]) * inv;
+  const bool store = xt < p.nx;
+  if (warp == 0) {
+    const double sax = (f(1) + f(2)) + (f(3) + f(4));
+    const double sdg = (f(5) + f(6)) + (f(7) + f(8));
+    const double rusq = rho * (ux * ux + uy * uy), uF = uy * Fy;
+    const double m1 = fma(2.0, sdg, -4.0 * f(0) - sax);
+    const double m2 = fma(-2.0, sax, fma(4.0, f(0), sdg));
+    const double he = 1.0 - 0.5 * p.s_e, heps = 1.0 - 0.5 * p.s_eps;
+    sm[A1][lane] = (1.0 / 36.0) *
+                   fma(-p.s_e, fma(-3.0, rusq, fma(2.0, drho, m1)), 6.0 * he * uF);
+    sm[A2][lane] = (1.0 / 36.0) * fma(-p.s_eps, fma(3.0, rusq, m2 - drho), -6.0 * heps * uF);
+    sm[A5][lane] = Fy * (1.0 / 6.0);
+  } else if (warp == 1) {
+    const double m4 = fma(-2.0, f(1) - f(3), (f(5) - f(6)) + (f(8) - f(7)));
+    const double m7 = (f(1) + f(3)) - (f(2) + f(4));
+    const double hnu = 1.0 - 0.5 * p.s_nu;
+    sm[A4][lane] = (1.0 / 12.0) * (-p.s_q * fma(rho, ux, m4));
+    sm[A7][lane] =
+        0.25 * fma(-p.s_nu, fma(rho, uy * uy - ux * ux, m7), -2.0 * hnu * (uy * Fy));
+  } else if (warp == 2) {
+    const double m6 = fma(-2.0, f(2) - f(4), (f(5) + f(6)) - (f(7) + f(8)));
+    const double m8 = (f(5) + f(7)) - (f(6) + f(8));
+    const double hq = 1.0 - 0.5 * p.s_q, hnu = 1.0 - 0.5 * p.s_nu;
+    sm[A6][lane] = (1.0 / 12.0) * fma(-p.s_q, fma(rho, uy, m6), -hq * Fy);
+    sm[A8][lane] = 0.25 * fma(-p.s_nu, m8 - rho * ux * uy, hnu * (ux * Fy));
+  } else {
+    const double n1 = g(1) - g(3), n2 = g(2) - g(4);
+    const double n3 = fma(-4.0, g(0), (g(1) + g(2)) + (g(3) + g(4)));
+    const double n4 = (g(1) + g(3)) - (g(2) + g(4));
+    const double b1 = -0.5 * p.q_j * (n1 - ux * Tr), b2 = -0.5 * p.q_j * (n2 - uy * Tr);
+    const double b3 = -0.05 * p.q_e * (n3 - p.a_T * Tr), b4 = -0.25 * p.q_nu * n4;
+    const double s34 = b3 + b4, d34 = b3 - b4;
+    if (store) {
+      double* o = fout + 9 * P + idx;
+      o[0] = fma(-4.0, b3, g(0));
+      o[P] = g(1) + (b1 + s34);
+      o[3 * P] = g(3) + (s34 - b1);
+      o[2 * P] = g(2) + (b2 + d34);
+      o[4 * P] = g(4) + (d34 - b2);
+    }
+  }
+  __syncthreads();
+  if (!store) return;
+  const double a1 = sm[A1][lane], a2 = sm[A2][lane];
+  double* o = fout + idx;
+  if (warp == 0) {
+    const double a4 = sm[A4][lane], t13 = fma(-2.0, a2, -a1) + sm[A7][lane];
+    o[0] = fma(4.0, a2 - a1, f(0));
+    o[P] = f(1) + fma(-2.0, a4, t13);
+    o[3 * P] = f(3) + fma(2.0, a4, t13);
+  } else if (warp == 1) {
+    const double t24 = fma(-2.0, a2, -a1) - sm[A7][lane];
+    const double v24 = fma(-2.0, sm[A6][lane], sm[A5][lane]);
+    o[2 * P] = f(2) + (t24 + v24);
+    o[4 * P] = f(4) + (t24 - v24);
+  } else {
+    const double cdg = fma(2.0, a1, a2), w56 = sm[A5][lane] + sm[A6][lane];
+    if (warp == 2) {
+      const double cp = cdg + w56, p48 = sm[A4][lane] + sm[A8][lane];
+      o[5 * P] = f(5) + (cp + p48);
+      o[6 * P] = f(6) + (cp - p48);
+    } else {
+      const double cm = cdg - w56, m48 = sm[A4][lane] - sm[A8][lane];
+      o[7 * P] = f(7) + (cm - m48);
+      o[8 * P] = f(8) + (cm + m48);
+    }
+  }
+}
+
 // Equilibrium (Sec. 2.1) of given fields, then the collision.  The flow
 // equilibrium is the second-order Hermite form w_i rho (1 + 3 e.u + 9/2 (e.u)^2
 // - 3/2 u^2), which has exactly the printed moments; the temperature
@@ -1368,6 +1511,18 @@ struct StepFn {
             case KV_TMA_R4S3: return launch_tma<S, 4, 3>(s, s.cur, out, p);
             default: break;
           }
+        }
+      }
+      if constexpr (std::is_same<S, double>::value) {
+        // up to two warps of k_step an SM: four times as many fit its schedulers
+        // (by the whole mesh: a slab computes the bits of the undivided one)
+        const dim3 grid((s.n[0] + 31) / 32, step_rows(s));
+        if ((long long)grid.x * s.n[1] <= 2LL * s.sm_count) {
+          if (s.uniform)
+            k_step_split<true><<<grid, 128, 0, s.stream>>>(in, out, p);
+          else
+            k_step_split<false><<<grid, 128, 0, s.stream>>>(in, out, p);
+          return cudaGetLastError();
         }
       }
       const int rows = step_block_rows(s);
