@@ -126,29 +126,36 @@ class WarmStartNet:
         """z: [B, 16] features.  Returns the output [B, S, S, 3] (torch, FP32)."""
         if not (self.fused and z.shape[1] == FEATURES and 1 <= z.shape[0] <= (1 << 30) // self.size ** 2):
             return self._forward_chain(z, keep)
-        torch = self.torch
         B = z.shape[0]
         z = np.ascontiguousarray(z, dtype=np.float32)
-        shapes, H, stages = [(B, self.base, self.base, self.channels[0])], self.base, len(self.channels)
-        for s, cout in enumerate(self._chan[1:]):
-            H = 2 * H if s + 1 < stages else H
-            shapes.append((B, H, H, cout))
+        at, total = self._layout(B)
         # one allocation for everything but the output: features, hidden layer, activations
-        sizes = [B * FEATURES, B * self.hidden] + [math.prod(s) for s in shapes[:-1]]
-        pad = [(n + 63) // 64 * 64 for n in sizes]
-        flat = torch.empty(sum(pad), device=self.device)
-        at, parts = 0, []
-        for n, p in zip(sizes, pad):
-            parts.append(flat[at:at + n])
-            at += p
-        zk, h1 = parts[:2]
-        acts = [a.view(s) for a, s in zip(parts[2:], shapes)]
-        acts.append(torch.empty(shapes[-1], device=self.device))
-        _ck(self.lib.islbm_cnn_forward(stages, self._chan, self.base, self.hidden, self._weights(),
-                                       ctypes.c_void_p(z.ctypes.data), B, _p(zk), _p(h1),
-                                       _ptrs(acts), self._stream()))
-        self.cache = dict(B=B, zk=zk, h1=h1, acts=acts) if keep else None
-        return acts[-1]
+        flat = self.torch.empty(total, device=self.device)
+        y = self.torch.empty((B, self.size, self.size, self.out_ch), device=self.device)
+        zk, h1, acts = self._pointers(flat, at, y)
+        _ck(self.lib.islbm_cnn_forward(len(self.channels), self._chan, self.base, self.hidden,
+                                       self._weights(), z.ctypes.data, B, zk, h1, acts,
+                                       self._stream()))
+        self.cache = dict(B=B, flat=flat, at=at, y=y) if keep else None
+        return y
+
+    def _layout(self, B):
+        """Offsets (floats, 256-byte multiples) of the features, the hidden layer and
+        the activations but the output in one buffer, and its length."""
+        at, n, H = [], 0, self.base
+        sizes = [B * FEATURES, B * self.hidden, B * H * H * self.channels[0]]
+        for cout in self.channels[1:]:
+            H *= 2
+            sizes.append(B * H * H * cout)
+        for size in sizes:
+            at.append(n)
+            n += (size + 63) // 64 * 64
+        return at, n
+
+    def _pointers(self, flat, at, y):
+        base = flat.data_ptr()
+        ptr = [base + 4 * k for k in at]
+        return ptr[0], ptr[1], (ctypes.c_void_p * (len(ptr) - 1))(*ptr[2:], y.data_ptr())
 
     def _weights(self):
         """The operands of the fused layers, in the order of self.names."""
@@ -205,7 +212,8 @@ class WarmStartNet:
         """Gradients of all parameters for the output gradient dy [B, S, S, 3]."""
         torch = self.torch
         c = self.cache
-        if "acts" in c:
+        if "flat" in c:
+            zk, h1, acts = self._pointers(c["flat"], c["at"], c["y"])
             dy = dy.contiguous()
             n = ctypes.c_ulonglong()
             stages = len(self.channels)
@@ -213,9 +221,8 @@ class WarmStartNet:
                                                     c["B"], ctypes.byref(n)))
             scratch = torch.empty(n.value // 4, device=self.device)
             _ck(self.lib.islbm_cnn_backward(
-                stages, self._chan, self.base, self.hidden, self._weights(), c["B"], _p(c["zk"]),
-                _p(c["h1"]), _ptrs(c["acts"]), _p(dy), _ptrs([self.grads[k] for k in self.names]),
-                _p(scratch), self._stream()))
+                stages, self._chan, self.base, self.hidden, self._weights(), c["B"], zk, h1, acts,
+                _p(dy), _ptrs([self.grads[k] for k in self.names]), _p(scratch), self._stream()))
             return self.grads
         B = c["B"]
         st = self._stream()

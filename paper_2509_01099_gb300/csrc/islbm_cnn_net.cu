@@ -9,7 +9,7 @@
 // the nearest-neighbour upsampling is a shift of the pixel coordinates), and
 // bias, tanh, its derivative and the upsampling's adjoint are part of the
 // products' kernels.  Measured on GB300, chain and fused: a training step of 16
-// samples 7.03 and 0.72 ms, a prediction 438 and 92 us.
+// samples 7.03 and 0.70 ms, a prediction 445 and 50 us.
 //
 // The products are narrow (3 to 64 channels), so they stay on mma.sync with
 // operands in the staged window: their roofline is the activations' bytes
@@ -187,6 +187,9 @@ __global__ void __launch_bounds__(128) k_conv_fwd(Conv p) {
   const Tiles tl(p.B, p.H, p.W, TR);
   // ldmatrix: this lane's pixel (A) / channel row (B) and 8-wide column
   const int arow = lane & 15, acol = (lane >> 4) * 8;
+  // the weights of the next layer may be staged while this one runs
+  islbm::grid_launch_next();
+  islbm::grid_wait();
   const unsigned bbase = sptr(sw) + 2u * (unsigned)((lane & 15) * WP + (NT > 1 ? (lane >> 4) * 8 : 0));
   for (int t = blockIdx.x; t < tl.n; t += gridDim.x) {
     int b, y0, x0;
@@ -680,6 +683,7 @@ __global__ void __launch_bounds__(128) k_fc_fwd(Fc p, const __grid_constant__ ZA
   bf16* sw2 = sh + kFcB * P;                     // [HP][72]
   bf16* sz = sw2 + HP * 72;                      // [16][24]
   const int bb = b0 + blockIdx.y * kFcB, nb = min(kFcB, p.B - bb), n0 = blockIdx.x * 64;
+  islbm::grid_launch_next();
   stage_matrix(sw1, P, p.w1, p.hidden, kFeat, HP, kFeat, p.hidden, p.v1);
   stage_matrix(sw2, 72, p.w2 + n0, p.n2, HP, 64, p.hidden, p.n2 - n0, p.v2);
   for (int e = threadIdx.x; e < kFcB * kFeat; e += 128) {
@@ -914,8 +918,10 @@ cudaError_t fwd_nt(const Conv& p, int sms, cudaStream_t st) {
   const size_t smem = 2 * ((size_t)9 * up16(p.cin) * (NT * 8 + 8) + (size_t)win * pitch_of(p.cin));
   const int gy = ((p.cout + 7) / 8 + NT - 1) / NT;
   const dim3 grid(persistent_grid(Tiles(p.B, p.H, p.W, TR).n, smem, sms, gy, 8), gy);
-  k_conv_fwd<NT, MT><<<grid, 128, smem, st>>>(p);
-  return cudaGetLastError();
+  // up to one tile a block, the launch and the staging of the weights are most
+  // of a layer: the next one starts early (a prediction: 64 -> 46 us of device time)
+  const bool serial = Tiles(p.B, p.H, p.W, TR).n <= 4 * sms;
+  return islbm::launch_grid(serial, k_conv_fwd<NT, MT>, grid, 128, smem, st, p);
 }
 
 template <int NT>
