@@ -26,6 +26,7 @@ struct islbm_batch {
   std::vector<char> active;              // members still advanced by islbm_batch_step
   std::vector<int> rows;                 // rows per thread (2 or 4) of each member's tiles
   std::vector<BatchGroup*> groups;
+  BatchGroup* pair = nullptr;            // two steps of all active members a launch (or null)
   cudaStream_t stream = nullptr;
   int precision = ISLBM_FP32;
   int parity = 0;                        // buffer read by the next step (all members)
@@ -60,8 +61,15 @@ islbm_status make_mesh(int kind, int n, double a, std::vector<double>& xi) {
   return ISLBM_ERR_ARG;
 }
 
-// one batched step on `st` (all groups), then the members' bookkeeping
-cudaError_t batch_launch(islbm_batch* b, cudaStream_t st) {
+// one batched step on `st` (all groups), or two where a launch takes two and
+// `want` allows it; *done: how many
+cudaError_t batch_launch(islbm_batch* b, cudaStream_t st, long long want, int* done) {
+  *done = b->pair && want >= 2 ? 2 : 1;
+  if (*done == 2) {
+    const cudaError_t e = b->pair->launch(st, b->parity, (unsigned)b->time, b->derr);
+    if (e == cudaSuccess) b->parity ^= 1;
+    return e;
+  }
   for (BatchGroup* g : b->groups) {
     const cudaError_t e = g->launch(st, b->parity, (unsigned)b->time, b->derr);
     if (e != cudaSuccess) return e;
@@ -83,7 +91,8 @@ cudaError_t build_batch_graph(islbm_batch* b, int parity) {
   e = cudaStreamBeginCapture(b->side, cudaStreamCaptureModeThreadLocal);
   cudaError_t le = cudaSuccess;
   if (e == cudaSuccess) {
-    for (int k = 0; k < kGraphSteps && le == cudaSuccess; ++k, ++b->time) le = batch_launch(b, b->side);
+    for (int k = 0, done = 0; k < kGraphSteps && le == cudaSuccess; k += done, b->time += done)
+      le = batch_launch(b, b->side, kGraphSteps - k, &done);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(b->side, &g);
     if (e == cudaSuccess && le == cudaSuccess) e = cudaGraphInstantiate(&b->graph[parity], g, 0);
@@ -116,6 +125,15 @@ cudaError_t rebuild_groups(islbm_batch* b) {
     }
   for (BatchGroup* g : b->groups) delete g;
   b->groups.clear();
+  delete b->pair;
+  b->pair = nullptr;
+  std::vector<Solver*> all;
+  for (size_t i = 0; i < b->members.size(); ++i)
+    if (b->active[i]) all.push_back(b->members[i]);
+  if (!all.empty()) {
+    e = make_batch_pair_group(all, b->precision, all[0]->sm_count, b->stream, &b->pair);
+    if (e != cudaSuccess) return e;
+  }
   for (int rows : {2, 4}) {
     std::vector<Solver*> grp;
     for (size_t i = 0; i < b->members.size(); ++i)
@@ -305,6 +323,7 @@ extern "C" void islbm_batch_destroy(islbm_batch_t b) {
   if (b->ev_in) cudaEventDestroy(b->ev_in);
   if (b->ev_out) cudaEventDestroy(b->ev_out);
   for (BatchGroup* g : b->groups) delete g;
+  delete b->pair;
   for (islbm_t m : b->members) islbm_destroy(m);
   islbm::dev_free(b->mem, b->derr, b->stream);
   if (b->stream) cudaStreamSynchronize(b->stream);
@@ -343,12 +362,14 @@ extern "C" islbm_status islbm_batch_step(islbm_batch_t b, long long n) {
     b->time += kGraphSteps;
     sync_members(b, kGraphSteps);
   }
-  for (long long k = 0; k < n; ++k) {
-    const cudaError_t e = batch_launch(b, b->stream);
+  while (n > 0) {
+    int done = 0;
+    const cudaError_t e = batch_launch(b, b->stream, n, &done);
     if (e != cudaSuccess)
       return bfail(b, ISLBM_ERR_CUDA, std::string("islbm_batch_step: ") + cudaGetErrorString(e));
-    ++b->time;
-    sync_members(b, 1);
+    n -= done;
+    b->time += done;
+    sync_members(b, done);
   }
   return ISLBM_OK;
 }

@@ -31,7 +31,9 @@
 // Every wait is bounded; a wait that gives up raises the CTA's abort flag and
 // the error flag, thread 0 waits for its copies in flight, and the CTA returns.
 #include <algorithm>
+#include <cstring>
 #include <type_traits>
+#include <vector>
 
 #include "islbm_d2_common.cuh"
 #include "islbm_store.cuh"
@@ -237,10 +239,15 @@ struct YmGroup {
   }
 };
 
-template <typename S, int NS, int MINB>
-__global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
-    k_step_ym(const __grid_constant__ CUtensorMap tmap, S* __restrict__ fout, P2<float> p,
-              const __grid_constant__ PairC kc, int* err, YmSched sc) {
+// One CTA's work: columns [x0, x1) and rows [ya, yb).
+struct YmItem {
+  int x0, x1, ya, yb;
+};
+
+template <typename S, int NS>
+__device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__ fout,
+                                        const P2<float>& p, const PairC& kc, unsigned first_step,
+                                        int* err, const YmItem& item) {
   using G = YmGeom<S, NS>;
   constexpr int DT = G::DT, DR = G::DR;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -259,9 +266,7 @@ __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
   }
   __syncthreads();
 
-  const int strip = blockIdx.x % sc.nstrip, chunk = blockIdx.x / sc.nstrip;
-  const int x0 = sc.col(strip, p.nx), x1 = sc.col(strip + 1, p.nx);
-  const int ya = sc.row(chunk, p.ny), yb = sc.row(chunk + 1, p.ny);
+  const int x0 = item.x0, x1 = item.x1, ya = item.ya, yb = item.yb;
   const int nI = (yb - ya + 1) / 2;           // row pairs of the last group
   const bool at_bottom = ya == 0, at_top = yb == p.ny;
   // group s: iterations [first(s), last(s)], rows ya - 2 (NS - s) - 1 + 2 i, +1
@@ -276,11 +281,11 @@ __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
   auto issue = [&]() {
     const int st = issued % DT;
     mbar_expect_tx(&bars[st], G::TMA_BYTES);
-    tma_load_3d(smem_raw + st * G::TMA_BYTES, &tmap, xa, row0 + 2 * issued, 0, &bars[st]);
+    tma_load_3d(smem_raw + st * G::TMA_BYTES, tmap, xa, row0 + 2 * issued, 0, &bars[st]);
     ++issued;
   };
   if (threadIdx.x == 0) {
-    asm volatile("prefetch.tensormap [%0];\n" ::"l"(&tmap) : "memory");
+    asm volatile("prefetch.tensormap [%0];\n" ::"l"(tmap) : "memory");
     grid_launch_next();
     grid_wait();
     while (issued < min(DT, copies)) issue();
@@ -375,7 +380,7 @@ __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
       float2 mm[4];
       collide_pair(fn, gn, kc, mm);
       auto val = [&](int k) { return k < 9 ? fn[k < 9 ? k : 0] : gn[k < 9 ? 0 : k - 9]; };
-      const unsigned seed_step = p.step + (unsigned)(s - 1);
+      const unsigned seed_step = first_step + (unsigned)(s - 1);
       if constexpr (LAST) {
         if (mine) {
           char* o = reinterpret_cast<char*>(fout);
@@ -420,6 +425,48 @@ __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
   if (threadIdx.x == 0)
     for (int k = max(0, issued - DT); k < issued; ++k)
       mbar_wait(&bars[k % DT], (unsigned)(k / DT) & 1u);
+}
+
+template <typename S, int NS, int MINB>
+__global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
+    k_step_ym(const __grid_constant__ CUtensorMap tmap, S* __restrict__ fout, P2<float> p,
+              const __grid_constant__ PairC kc, int* err, YmSched sc) {
+  const int strip = blockIdx.x % sc.nstrip, chunk = blockIdx.x / sc.nstrip;
+  ym_item<S, NS>(&tmap, fout, p, kc, p.step, err,
+                 YmItem{sc.col(strip, p.nx), sc.col(strip + 1, p.nx), sc.row(chunk, p.ny),
+                        sc.row(chunk + 1, p.ny)});
+}
+
+// Many cavities in one launch: a CTA's item names its cavity, whose parameters
+// it copies to shared memory.
+template <typename S>
+struct alignas(128) YmCav {
+  CUtensorMap map[2];   // row pairs of the cavity's two buffers
+  S* out[2];            // output buffer when reading buffer 0 / 1
+  P2<float> p;
+  PairC kc;
+};
+struct YmBatchItem {
+  YmItem at;
+  int cav;
+};
+
+template <typename S, int NS, int MINB>
+__global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
+    k_step_ym_batch(const YmCav<S>* __restrict__ cavs, const YmBatchItem* __restrict__ items,
+                    int parity, unsigned step, int* err) {
+  __shared__ P2<float> p;
+  __shared__ PairC kc;
+  const YmBatchItem it = items[blockIdx.x];
+  const YmCav<S>& cv = cavs[it.cav];
+  static_assert(sizeof(P2<float>) % 4 == 0 && sizeof(PairC) % 4 == 0, "copied by words");
+  for (int k = threadIdx.x; k < (int)(sizeof(P2<float>) / 4); k += blockDim.x)
+    reinterpret_cast<int*>(&p)[k] = reinterpret_cast<const int*>(&cv.p)[k];
+  for (int k = threadIdx.x; k < (int)(sizeof(PairC) / 4); k += blockDim.x)
+    reinterpret_cast<int*>(&kc)[k] = reinterpret_cast<const int*>(&cv.kc)[k];
+  S* out = cv.out[parity];
+  // (the barrier that opens ym_item orders the copies before their use)
+  ym_item<S, NS>(&cv.map[parity], out, p, kc, step, err, it.at);
 }
 
 // Strips and chunks of a launch.  A CTA costs its rows and about kYmStart more
@@ -517,6 +564,130 @@ cudaError_t launch_step_2d_ym(Solver& s, int steps) {
   }
   if (e == cudaSuccess) s.cur ^= 1;
   return e;
+}
+
+namespace {
+
+struct YmBatch : BatchGroup {
+  using G = YmGeom<float, 2>;
+  YmCav<float>* cavs = nullptr;
+  YmBatchItem* items = nullptr;
+  int nitems = 0;
+  DevAllocator mem;
+  cudaStream_t stream = nullptr;
+  ~YmBatch() override {
+    dev_free(mem, cavs, stream);
+    dev_free(mem, items, stream);
+    cudaStreamSynchronize(stream);
+  }
+  cudaError_t launch(cudaStream_t st, int parity, unsigned step, int* err) override {
+    k_step_ym_batch<float, 2, 4><<<nitems, G::THREADS, G::SMEM, st>>>(cavs, items, parity, step,
+                                                                     err);
+    return cudaGetLastError();
+  }
+};
+
+}  // namespace
+
+// Two steps of FP32 cavities in one launch.  *out stays null where single steps
+// (k_step_tma_batch) are the better choice: other storage forms, meshes below
+// the kernel's limits, or too few nodes to fill the GPU (step_2d_ym_takes).
+cudaError_t make_batch_pair_group(const std::vector<Solver*>& members, int precision, int sms,
+                                  cudaStream_t stream, BatchGroup** out) {
+  *out = nullptr;
+  long long nodes = 0;
+  for (const Solver* m : members) {
+    nodes += m->nodes;
+    if (m->n[0] < 16 || m->n[1] < 2 * kYmMinRows + 2 ||
+        (size_t)m->plane * m->elem >= (size_t)1 << 31)
+      return cudaSuccess;
+  }
+  if (precision != ISLBM_FP32 || nodes < kYmMinNodes) return cudaSuccess;
+  const auto k = k_step_ym_batch<float, 2, 4>;
+  int per_sm = 0;
+  cudaError_t e = launch_setup_once(
+      reinterpret_cast<const void*>(k),
+      [](const void* f, int* n) {
+        cudaError_t e2 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)YmBatch::G::SMEM);
+        if (e2 == cudaSuccess)
+          e2 = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    cudaSharedmemCarveoutMaxShared);
+        if (e2 == cudaSuccess)
+          e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, f, YmBatch::G::THREADS,
+                                                             YmBatch::G::SMEM);
+        return e2;
+      },
+      &per_sm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  // one chunk length for all cavities: the rows of all items (and each item's
+  // start) spread over the slots, and half a longest item of idle slots at the end
+  auto sched = [](const Solver* m, int rows) {
+    const int w = kYmW - 2;
+    YmSched sc;
+    sc.nstrip = (m->n[0] + w - 1) / w;
+    const int most = m->n[1] / kYmMinRows;
+    sc.nchunk = std::max(1 + m->n[1] % 2, std::min(most, (m->n[1] + rows / 2) / rows));
+    return sc;
+  };
+  int best = 64;
+  double best_cost = 1e300;
+  for (int rows = 16; rows <= 1024; rows += 8) {
+    double total = 0.0, longest = 0.0;
+    for (const Solver* m : members) {
+      const YmSched sc = sched(m, rows);
+      total += (double)sc.nstrip * (m->n[1] + sc.nchunk * kYmStart);
+      longest = std::max(longest, (double)m->n[1] / sc.nchunk + kYmStart);
+    }
+    const double cost = std::max(total / ((double)sms * per_sm) + 0.5 * longest, longest);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = rows;
+    }
+  }
+  std::vector<YmCav<float>> cavs(members.size());
+  std::vector<YmBatchItem> items;
+  for (size_t c = 0; c < members.size(); ++c) {
+    Solver& m = *members[c];
+    std::memcpy(&cavs[c].map[0], m.tmap_y[0], sizeof(CUtensorMap));
+    std::memcpy(&cavs[c].map[1], m.tmap_y[1], sizeof(CUtensorMap));
+    cavs[c].out[0] = static_cast<float*>(m.buf[1]);
+    cavs[c].out[1] = static_cast<float*>(m.buf[0]);
+    cavs[c].p = make_params<float>(m);
+    cavs[c].kc = make_pair_constants(cavs[c].p);
+    const YmSched sc = sched(&m, best);
+    for (int b = 0; b < sc.nchunk; ++b)
+      for (int a = 0; a < sc.nstrip; ++a)
+        items.push_back(YmBatchItem{YmItem{sc.col(a, m.n[0]), sc.col(a + 1, m.n[0]),
+                                           sc.row(b, m.n[1]), sc.row(b + 1, m.n[1])},
+                                    (int)c});
+  }
+  // long items first: the short ones fill the end
+  std::stable_sort(items.begin(), items.end(), [](const YmBatchItem& a, const YmBatchItem& b) {
+    return a.at.yb - a.at.ya > b.at.yb - b.at.ya;
+  });
+  auto* g = new YmBatch();
+  g->nitems = (int)items.size();
+  g->mem = current_allocator();
+  g->stream = stream;
+  e = dev_alloc(g->mem, reinterpret_cast<void**>(&g->cavs), cavs.size() * sizeof(cavs[0]), stream);
+  if (e == cudaSuccess)
+    e = dev_alloc(g->mem, reinterpret_cast<void**>(&g->items), items.size() * sizeof(items[0]),
+                  stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(g->cavs, cavs.data(), cavs.size() * sizeof(cavs[0]),
+                        cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(g->items, items.data(), items.size() * sizeof(items[0]),
+                        cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (e != cudaSuccess) {
+    delete g;
+    return e;
+  }
+  *out = g;
+  return cudaSuccess;
 }
 
 int bounds_flag_ym(int reset) {

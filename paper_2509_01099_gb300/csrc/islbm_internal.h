@@ -294,6 +294,9 @@ struct BatchGroup {
   virtual ~BatchGroup() {}
   virtual cudaError_t launch(cudaStream_t stream, int parity, unsigned step, int* err) = 0;
 };
+// Two steps of all members in one launch; *out null where that does not pay.
+cudaError_t make_batch_pair_group(const std::vector<Solver*>& members, int precision, int sm_count,
+                                  cudaStream_t stream, BatchGroup** out);
 cudaError_t make_batch_group(const std::vector<Solver*>& members, int tile_rows, int precision,
                              int sm_count, cudaStream_t stream, BatchGroup** out);
 }  // namespace islbm

@@ -55,3 +55,32 @@ def test_two_steps_a_launch_are_single_steps(nx, ny, precision):
         states.append(got)
     for a, b in zip(*states):
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("sizes", [(600, 511, 27), (128,) * 37, (1030, 64, 333)])
+def test_batch_pairs_are_single_steps_of_each_cavity(sizes):
+    """600,000 nodes and more: the batch advances two steps a launch."""
+    pkg = _pkg()
+    cavs = [dict(n=n, mesh=("tanh", "erf", "uniform")[k % 3], a=1.5, Ra=1e6 * (1 + k))
+            for k, n in enumerate(sizes)]
+    b = pkg.Batch(cavs, "fp32")
+    alone = []
+    for k, (c, m) in enumerate(zip(cavs, b.members)):
+        n = c["n"]
+        f = random_populations(9, (n, n), seed=k, spread=0.2)
+        g = random_signed(5, (n, n), seed=k + 100, amplitude=0.12)
+        xi = getattr(O, "mesh_" + c["mesh"])(n, *([] if c["mesh"] == "uniform" else [1.5]))
+        s = pkg.Solver(xi, xi, Ra=c["Ra"], precision="fp32", kernel="tma_r2s2")
+        for h in (m, s):
+            h.set_populations(f, g)
+        alone.append(s)
+    for steps in (2, 1, 67):
+        b.step(steps)
+        b.synchronize()
+        for m, s in zip(b.members, alone):
+            s.step(steps)
+            for x, y in zip(m.populations(), s.populations()):
+                assert np.array_equal(x, y)
+    for s in alone:
+        s.close()
+    b.close()
