@@ -219,16 +219,23 @@ std::string encode_tensor_maps(Solver* s) {
         return "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
     } else {
       std::memcpy(s->tmap_m[b], s->tmap[b], sizeof(s->tmap_m[b]));
-      unsigned yb[3];
-      step_2d_ym_box((int)s->elem, yb);
-      const cuuint32_t ybox[3] = {yb[0], yb[1], yb[2]};
-      r = reinterpret_cast<EncodeFn>(fn)(
-          reinterpret_cast<CUtensorMap*>(s->tmap_y[b]), dt, 3, s->buf[b], dims, strides, ybox, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (r != CUDA_SUCCESS)
-        return "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
     }
+    // row pairs of the marching kernel
+    unsigned yb[3], ym[3];
+    step_2d_ym_box(s->precision, yb, ym);
+    const cuuint32_t ybox[3] = {yb[0], yb[1], yb[2]}, ymbox[3] = {ym[0], ym[1], ym[2]};
+    r = reinterpret_cast<EncodeFn>(fn)(
+        reinterpret_cast<CUtensorMap*>(s->tmap_y[b]), dt, 3, s->buf[b], dims, strides, ybox, estr,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r == CUDA_SUCCESS && s->precision == ISLBM_FP16NEQ)
+      r = reinterpret_cast<EncodeFn>(fn)(
+          reinterpret_cast<CUtensorMap*>(s->tmap_ym[b]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, mbase,
+          mdims, mstrides, ymbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    else
+      std::memcpy(s->tmap_ym[b], s->tmap_y[b], sizeof(s->tmap_ym[b]));
+    if (r != CUDA_SUCCESS) return "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
   }
   return "";
 }
@@ -580,8 +587,7 @@ extern "C" islbm_status islbm_create(const double* xi_x, int nx, const double* x
   // two steps a launch where the library chose the kernel (a variant that the
   // caller named runs as named)
   s->marching = dim == 2 && prm.kernel == KV_AUTO && s->variant >= KV_TMA_R4S2 &&
-                precision != ISLBM_FP16NEQ &&
-                step_2d_ym_takes(s->n[0], s->n[1], (int)s->elem, (size_t)s->plane * s->elem);
+                step_2d_ym_takes(s->n[0], s->n[1], precision, (size_t)s->plane * s->elem);
   // FP16NEQ: 14 planes of FP16 remainders, then 4 planes of FP32 moments
   s->state_bytes = precision == ISLBM_FP16NEQ
                        ? (size_t)s->plane * (14 * 2 + 4 * 4)

@@ -1,12 +1,15 @@
 // Marching 2-D step kernel: several time steps in one pass over the state
-// (Sec. 2.1 - 2.3; FP32 and 16-bit deviation storage, node-centred stencil).
+// (Sec. 2.1 - 2.3; FP32 and the 16-bit storage forms, node-centred stencil).
 //
 // A CTA owns a strip of up to 64 - 2 (NS - 1) columns over a chunk of rows and
 // marches through it two rows at a time.  NS groups of two warps work as a
 // pipeline: group s computes time step s of the rows that group s - 1 has just
 // finished (group 1 reads rows brought by TMA) and hands its rows on through a
 // ring in shared memory; only the last group writes to global memory.  A thread
-// keeps one column for the whole chunk.
+// keeps one column for the whole chunk.  In the FP16NEQ form one more group in
+// front decodes every staged row once (the tile kernel decodes 1.4 rows for a
+// row of results, between two CTA-wide barriers), and the rows handed on are
+// encoded and decoded again in registers.
 //
 // Why.  The tile kernel (k_step_tma) moves the whole state through HBM once a
 // step and needs 324 instructions a node, many of them twice: it interpolates
@@ -47,21 +50,31 @@ constexpr int kYmMinRows = 12;     // shortest chunk
 
 template <typename S, int NS>
 struct YmGeom {
+  // FP16NEQ: one more group in front decodes the staged rows into a ring
+  static constexpr bool NEQ = is_neq<S>::value;
+  static constexpr int LEVELS = NS + (NEQ ? 1 : 0), RINGS = LEVELS - 1;
+  static constexpr int COLUMNS = kYmW - 2 * (LEVELS - 1);   // widest strip
   static constexpr int HX = 16 / (int)sizeof(S);       // elements of a 16-byte chunk
-  // staged row: the columns of group 1 with one halo column on each side, from
-  // a 16-byte boundary
-  static constexpr int TW = (kYmW + 2 + HX - 1 + HX - 1) / HX * HX;
+  // staged row: the columns of the first group, with one halo column on each
+  // side where it interpolates, from a 16-byte boundary
+  static constexpr int TW = (kYmW + (NEQ ? 0 : 2) + HX - 1 + HX - 1) / HX * HX;
+  static constexpr int MW = (kYmW + 3 + 3) / 4 * 4;    // FP16NEQ: row of the FP32 moments
   // row pitch of the rings between groups, whose rows are FP32 in every storage
   // form (rounded to it, so that the next group reads them without conversions)
   static constexpr int RW = kYmW + 2;
-  static constexpr unsigned TMA_BYTES = 14u * 2u * TW * sizeof(S);
+  static constexpr unsigned ROWS = 14u * 2u * TW * sizeof(S);
+  static constexpr unsigned M_OFF = (ROWS + 127u) / 128u * 128u;
+  static constexpr unsigned M_BYTES = NEQ ? 4u * 2u * MW * 4u : 0u;
+  static constexpr unsigned LOADED = ROWS + M_BYTES;   // bytes a stage's copies bring
+  static constexpr unsigned TMA_BYTES = M_OFF + M_BYTES;
   static constexpr unsigned RING_BYTES = (14u * 2u * RW * 4u + 127u) / 128u * 128u;
   static constexpr int DT = 3;                         // TMA stages (row pairs)
-  static constexpr int DR = 4;                         // row pairs of a ring
-  static constexpr unsigned SMEM = DT * TMA_BYTES + (NS - 1) * DR * RING_BYTES + 256;
-  static constexpr int THREADS = NS * 64;
+  static constexpr int DR = 4;               // row pairs of a ring
+  static constexpr unsigned SMEM = DT * TMA_BYTES + RINGS * DR * RING_BYTES + 256;
+  static constexpr int THREADS = LEVELS * 64;
+  static constexpr int CTAS = NEQ ? 2 : NS == 2 ? 4 : 6;   // an SM's registers and shared memory
   static_assert(TMA_BYTES % 128 == 0, "stages keep the TMA's 128-byte alignment");
-  static_assert((2 * DT + 2 * DR * (NS - 1)) * 8 + 4 <= 256 - 16, "barriers and the flag");
+  static_assert((2 * DT + 2 * DR * RINGS) * 8 + 4 <= 256 - 16, "barriers and the flag");
 };
 
 // The items of a launch: strips of columns x chunks of rows, evenly split.
@@ -101,9 +114,11 @@ __device__ __forceinline__ void ym_wait(uint64_t* bar, unsigned phase, volatile 
 template <typename S, int NS, int s>
 struct YmGroup {
   using G = YmGeom<S, NS>;
+  using Elem = S;
   static constexpr bool FIRST = s == 1, LAST = s == NS;
-  using T = std::conditional_t<FIRST, S, float>;       // type of the source rows
-  static constexpr int RS = FIRST ? G::TW : G::RW;     // row pitch of the source
+  static constexpr bool STAGED = FIRST && !G::NEQ;     // source: the TMA stages
+  using T = std::conditional_t<STAGED, S, float>;      // type of the source rows
+  static constexpr int RS = STAGED ? G::TW : G::RW;    // row pitch of the source
   static constexpr int PS = 2 * RS;                    // plane pitch of the source
 
   // per-thread state of the march
@@ -245,22 +260,22 @@ struct YmItem {
 };
 
 template <typename S, int NS>
-__device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__ fout,
-                                        const P2<float>& p, const PairC& kc, unsigned first_step,
+__device__ __forceinline__ void ym_item(const CUtensorMap* tmap, const CUtensorMap* tmap_m,
+                                        S* __restrict__ fout, const P2<float>& p, const PairC& kc, unsigned first_step,
                                         int* err, const YmItem& item) {
   using G = YmGeom<S, NS>;
-  constexpr int DT = G::DT, DR = G::DR;
+  constexpr int DT = G::DT, DR = G::DR, RINGS = G::RINGS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* rings = smem_raw + DT * G::TMA_BYTES;
   // full / empty barriers of the TMA stages, then of each ring
-  uint64_t* bars = reinterpret_cast<uint64_t*>(rings + (NS - 1) * DR * G::RING_BYTES + 16);
-  volatile int* abort = reinterpret_cast<volatile int*>(bars + 2 * DT + 2 * DR * (NS - 1));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(rings + RINGS * DR * G::RING_BYTES + 16);
+  volatile int* abort = reinterpret_cast<volatile int*>(bars + 2 * DT + 2 * DR * RINGS);
   if (threadIdx.x == 0) {
     for (int k = 0; k < DT; ++k) {
       mbar_init(&bars[k], 1);
       mbar_init(&bars[DT + k], 2);
     }
-    for (int k = 0; k < 2 * DR * (NS - 1); ++k) mbar_init(&bars[2 * DT + k], 2);
+    for (int k = 0; k < 2 * DR * RINGS; ++k) mbar_init(&bars[2 * DT + k], 2);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -280,8 +295,11 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__
   int issued = 0;
   auto issue = [&]() {
     const int st = issued % DT;
-    mbar_expect_tx(&bars[st], G::TMA_BYTES);
-    tma_load_3d(smem_raw + st * G::TMA_BYTES, tmap, xa, row0 + 2 * issued, 0, &bars[st]);
+    unsigned char* dst = smem_raw + st * G::TMA_BYTES;
+    mbar_expect_tx(&bars[st], G::LOADED);
+    tma_load_3d(dst, tmap, xa, row0 + 2 * issued, 0, &bars[st]);
+    if constexpr (G::NEQ)
+      tma_load_3d(dst + G::M_OFF, tmap_m, (x0 - NS) & ~3, row0 + 2 * issued, 0, &bars[st]);
     ++issued;
   };
   if (threadIdx.x == 0) {
@@ -290,32 +308,91 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__
     grid_wait();
     while (issued < min(DT, copies)) issue();
   }
+  // Refill of the stage of the iteration before, which the other warp has
+  // released by now or does within this iteration.
+  auto refill = [&]() {
+    const int u = issued - DT;
+    ym_wait(&bars[DT + u % DT], (unsigned)(u / DT) & 1u, abort, err);
+    if (!*abort) {
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      issue();
+    }
+  };
+  // FP16NEQ: the staged row pairs as FP32 deviations, one column a thread.
+  [[maybe_unused]] auto decode = [&]() {
+    if constexpr (G::NEQ) {
+      const int x = x0 - NS + (int)threadIdx.x;
+      const int hc = x - xa, mc = x - ((x0 - NS) & ~3);
+      uint64_t* tfull = bars + 2 * DT;
+      uint64_t* tempty = tfull + DR;
+      float t0, ti;
+      trest(p.a_T, t0, ti);
+      int ss = 0, ts = 0;
+      unsigned sp = 0, tp = 1;
+      for (int n = 0; n < copies; ++n) {
+        ym_wait(&bars[ss], sp, abort, err);
+        const unsigned char* stage = smem_raw + ss * G::TMA_BYTES;
+        const unsigned short* h = reinterpret_cast<const unsigned short*>(stage) + hc;
+        const float* m = reinterpret_cast<const float*>(stage + G::M_OFF) + mc;
+        unsigned r[14];
+#pragma unroll
+        for (int k = 0; k < 14; ++k)
+          r[k] = (unsigned)h[2 * k * G::TW] | ((unsigned)h[(2 * k + 1) * G::TW] << 16);
+        float2 mm[4], f[9], g[5];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mm[k] = make_float2(m[2 * k * G::MW], m[(2 * k + 1) * G::MW]);
+        neq_decode2x2(mm[0], mm[1], mm[2], mm[3], r, t0, ti, f, g);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars[DT + ss]);
+        if (threadIdx.x == 0 && n > 0 && issued < copies) refill();
+        ym_wait(&tempty[ts], tp, abort, err);
+        float* t = reinterpret_cast<float*>(rings + ts * G::RING_BYTES) + threadIdx.x;
+#pragma unroll
+        for (int k = 0; k < 14; ++k) {
+          const float2 v = k < 9 ? f[k < 9 ? k : 0] : g[k < 9 ? 0 : k - 9];
+          t[2 * k * G::RW] = v.x;
+          t[(2 * k + 1) * G::RW] = v.y;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tfull[ts]);
+        if (++ss == DT) {
+          ss = 0;
+          sp ^= 1u;
+        }
+        if (++ts == DR) {
+          ts = 0;
+          tp ^= 1u;
+        }
+      }
+    }
+  };
   auto run = [&](auto step) {
     constexpr int s = decltype(step)::value;
     using Gr = YmGroup<S, NS, s>;
     using T = typename Gr::T;
-    constexpr bool FIRST = Gr::FIRST, LAST = Gr::LAST;
-    const int c = threadIdx.x - 64 * (s - 1);
+    using St = Store<typename Gr::Elem>;
+    constexpr bool FIRST = Gr::FIRST, LAST = Gr::LAST, STAGED = Gr::STAGED;
+    constexpr int RT = G::NEQ ? s : s - 1;    // ring written; RT - 1: ring read
+    const int c = threadIdx.x - 64 * RT;
     const int x = x0 - (NS - s) + c;
-    const int src0 = FIRST ? xa : x0 - NS + s - 1;
+    const int src0 = STAGED ? xa : x0 - NS + s - 1;
     Gr g;
     g.setup(p, x, src0);
-    // source: the TMA stages or ring s - 2 (between groups s - 1 and s); target: ring s - 1
-    uint64_t* sfull = FIRST ? bars : bars + 2 * DT + 2 * DR * (s - 2);
-    uint64_t* sempty = sfull + (FIRST ? DT : DR);
-    uint64_t* tfull = bars + 2 * DT + 2 * DR * (s - 1);
+    uint64_t* sfull = STAGED ? bars : bars + 2 * DT + 2 * DR * (RT - 1);
+    uint64_t* sempty = sfull + (STAGED ? DT : DR);
+    uint64_t* tfull = bars + 2 * DT + 2 * DR * RT;
     uint64_t* tempty = tfull + DR;
-    constexpr int DS = FIRST ? DT : DR;
-    const unsigned char* src = FIRST ? smem_raw : rings + (s - 2) * DR * G::RING_BYTES;
-    constexpr unsigned SB = FIRST ? G::TMA_BYTES : G::RING_BYTES;
-    unsigned char* target = rings + (s - 1) * DR * G::RING_BYTES;
+    constexpr int DS = STAGED ? DT : DR;
+    const unsigned char* src = STAGED ? smem_raw : rings + (RT - 1) * DR * G::RING_BYTES;
+    constexpr unsigned SB = STAGED ? G::TMA_BYTES : G::RING_BYTES;
+    unsigned char* target = rings + RT * DR * G::RING_BYTES;
     const int i0 = first(s), i1 = last(s);
     const bool mine = x >= x0 && x < x1;
     int ss = 0;              // source slot of this iteration's (first) row pair
     unsigned sp = 0;         // its phase
     int ts = 0;              // target slot
     unsigned tp = 1;         // phase of its empty barrier (1: the first use passes)
-    // source rows of iteration i: FIRST: both of stage ss; else the second row of
+    // source rows of iteration i: FIRST: both of slot ss; else the second row of
     // pair i (slot ss) and the first row of pair i + 1 (the next slot)
     if (!FIRST && !at_bottom) ym_wait(&sfull[0], 0u, abort, err);
     // a bottom chunk has no pair i0: its first pair is taken as "next"
@@ -356,16 +433,7 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__
       // the source rows are in registers: release stage / pair i
       __syncwarp();
       if (have && lane == 0) mbar_arrive(&sempty[ss]);
-      if (FIRST && threadIdx.x == 0 && i > i0 && issued < copies) {
-        // refill the stage of the iteration before, which the other warp has
-        // released by now (or does within this iteration)
-        const int n = issued - DT;
-        ym_wait(&sempty[n % DT], (unsigned)(n / DT) & 1u, abort, err);
-        if (!*abort) {
-          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-          issue();
-        }
-      }
+      if (STAGED && threadIdx.x == 0 && i > i0 && issued < copies) refill();
       if (FIRST) {
         if (++ss == DS) {
           ss = 0;
@@ -381,32 +449,68 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__
       collide_pair(fn, gn, kc, mm);
       auto val = [&](int k) { return k < 9 ? fn[k < 9 ? k : 0] : gn[k < 9 ? 0 : k - 9]; };
       const unsigned seed_step = first_step + (unsigned)(s - 1);
-      if constexpr (LAST) {
+      [[maybe_unused]] unsigned rr[14];   // FP16NEQ: remainders of rows R - 1 (low halves) and R
+      [[maybe_unused]] float t0, ti;
+      if constexpr (G::NEQ) {
+        trest(p.a_T, t0, ti);
+        neq_remainders2x2(fn, gn, mm, t0, ti, rr);
+      }
+      if constexpr (LAST && G::NEQ) {
+        if (mine) {
+          char* o = reinterpret_cast<char*>(fout);
+          const size_t ps = (size_t)p.plane * 2;
+          char* om = o + 14 * ps;
+#pragma unroll
+          for (int k = 0; k < 14; ++k)
+            *reinterpret_cast<unsigned short*>(o + k * ps + off) = (unsigned short)(rr[k] & 0xFFFFu);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) *reinterpret_cast<float*>(om + 2 * (k * ps + off)) = mm[k].x;
+          if (R < yb) {
+            const size_t off1 = off + (size_t)p.pitch * 2;
+#pragma unroll
+            for (int k = 0; k < 14; ++k)
+              *reinterpret_cast<unsigned short*>(o + k * ps + off1) = (unsigned short)(rr[k] >> 16);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              *reinterpret_cast<float*>(om + 2 * (k * ps + off1)) = mm[k].y;
+          }
+        }
+        off += (unsigned)(2 * p.pitch * sizeof(S));
+      } else if constexpr (LAST) {
         if (mine) {
           char* o = reinterpret_cast<char*>(fout);
           const size_t ps = (size_t)p.plane * sizeof(S);
           unsigned r = sr_seed((size_t)(R - 1) * p.pitch + x, seed_step);
 #pragma unroll
           for (int k = 0; k < 14; ++k)
-            Store<S>::st_sr(reinterpret_cast<S*>(o + k * ps + off), val(k).x, sr_next(r));
+            St::st_sr(reinterpret_cast<S*>(o + k * ps + off), val(k).x, sr_next(r));
           if (R < yb) {
             const unsigned off1 = off + (unsigned)(p.pitch * sizeof(S));
             unsigned r1 = sr_seed((size_t)R * p.pitch + x, seed_step);
 #pragma unroll
             for (int k = 0; k < 14; ++k)
-              Store<S>::st_sr(reinterpret_cast<S*>(o + k * ps + off1), val(k).y, sr_next(r1));
+              St::st_sr(reinterpret_cast<S*>(o + k * ps + off1), val(k).y, sr_next(r1));
           }
         }
         off += (unsigned)(2 * p.pitch * sizeof(S));
       } else {
         ym_wait(&tempty[ts], tp, abort, err);
         float* t = reinterpret_cast<float*>(target + ts * G::RING_BYTES) + c;
-        unsigned r = sr_seed((size_t)((long long)(R - 1) * p.pitch + x), seed_step);
-        unsigned r1 = sr_seed((size_t)((long long)R * p.pitch + x), seed_step);
+        if constexpr (G::NEQ) {   // what the next step would read back
+          neq_decode2x2(mm[0], mm[1], mm[2], mm[3], rr, t0, ti, fn, gn);
 #pragma unroll
-        for (int k = 0; k < 14; ++k) {
-          t[k * 2 * G::RW] = Store<S>::rounded_sr(val(k).x, sr_next(r));
-          t[k * 2 * G::RW + G::RW] = Store<S>::rounded_sr(val(k).y, sr_next(r1));
+          for (int k = 0; k < 14; ++k) {
+            t[k * 2 * G::RW] = val(k).x;
+            t[k * 2 * G::RW + G::RW] = val(k).y;
+          }
+        } else {
+          unsigned r = sr_seed((size_t)((long long)(R - 1) * p.pitch + x), seed_step);
+          unsigned r1 = sr_seed((size_t)((long long)R * p.pitch + x), seed_step);
+#pragma unroll
+          for (int k = 0; k < 14; ++k) {
+            t[k * 2 * G::RW] = St::rounded_sr(val(k).x, sr_next(r));
+            t[k * 2 * G::RW + G::RW] = St::rounded_sr(val(k).y, sr_next(r1));
+          }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&tfull[ts]);
@@ -417,7 +521,10 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__
       }
     }
   };
-  if (warp < 2)
+  constexpr int front = G::NEQ ? 2 : 0;    // warps of the decoding group
+  if (warp < front)
+    decode();
+  else if (warp < front + 2)
     run(std::integral_constant<int, 1>{});
   else if constexpr (NS > 1)
     run(std::integral_constant<int, 2>{});
@@ -429,10 +536,11 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, S* __restrict__
 
 template <typename S, int NS, int MINB>
 __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
-    k_step_ym(const __grid_constant__ CUtensorMap tmap, S* __restrict__ fout, P2<float> p,
-              const __grid_constant__ PairC kc, int* err, YmSched sc) {
+    k_step_ym(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_m,
+              S* __restrict__ fout, P2<float> p, const __grid_constant__ PairC kc, int* err,
+              YmSched sc) {
   const int strip = blockIdx.x % sc.nstrip, chunk = blockIdx.x / sc.nstrip;
-  ym_item<S, NS>(&tmap, fout, p, kc, p.step, err,
+  ym_item<S, NS>(&tmap, &tmap_m, fout, p, kc, p.step, err,
                  YmItem{sc.col(strip, p.nx), sc.col(strip + 1, p.nx), sc.row(chunk, p.ny),
                         sc.row(chunk + 1, p.ny)});
 }
@@ -466,7 +574,7 @@ __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
     reinterpret_cast<int*>(&kc)[k] = reinterpret_cast<const int*>(&cv.kc)[k];
   S* out = cv.out[parity];
   // (the barrier that opens ym_item orders the copies before their use)
-  ym_item<S, NS>(&cv.map[parity], out, p, kc, step, err, it.at);
+  ym_item<S, NS>(&cv.map[parity], nullptr, out, p, kc, step, err, it.at);
 }
 
 // Strips and chunks of a launch.  A CTA costs its rows and about kYmStart more
@@ -478,10 +586,8 @@ __global__ void __launch_bounds__(YmGeom<S, NS>::THREADS, MINB)
 constexpr double kYmStart = 8.0;
 constexpr double kYmRow[5] = {0.0, 0.25, 0.30, 0.345, 0.42};
 
-template <int NS>
-YmSched ym_schedule(int nx, int ny, int sms, int per_sm) {
+inline YmSched ym_schedule(int nx, int ny, int w, int sms, int per_sm) {
   YmSched sc;
-  const int w = kYmW - 2 * (NS - 1);
   sc.nstrip = (nx + w - 1) / w;
   sc.nchunk = 1;
   double best = 1e300;
@@ -502,8 +608,7 @@ YmSched ym_schedule(int nx, int ny, int sms, int per_sm) {
 template <typename S, int NS>
 cudaError_t launch_ym(Solver& s) {
   using G = YmGeom<S, NS>;
-  constexpr int MINB = NS == 2 ? 4 : 6;
-  const auto k = k_step_ym<S, NS, MINB>;
+  const auto k = k_step_ym<S, NS, G::CTAS>;
   int per_sm = 0;
   const cudaError_t e = launch_setup_once(
       reinterpret_cast<const void*>(k),
@@ -520,7 +625,7 @@ cudaError_t launch_ym(Solver& s) {
       &per_sm);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const YmSched sc = ym_schedule<NS>(s.n[0], s.n[1], s.sm_count, per_sm);
+  const YmSched sc = ym_schedule(s.n[0], s.n[1], G::COLUMNS, s.sm_count, per_sm);
   const P2<float> p = make_params<float>(s);
   // a launch that fills the GPU's slots leaves the next one's early blocks only
   // those that come free; into a half-full GPU they would crowd on the SMs with
@@ -529,6 +634,7 @@ cudaError_t launch_ym(Solver& s) {
   const bool serial = sc.nstrip * sc.nchunk >= s.sm_count * per_sm * 15 / 16;
   return launch_grid(serial, k, sc.nstrip * sc.nchunk, G::THREADS, G::SMEM, s.stream,
                      *reinterpret_cast<const CUtensorMap*>(s.tmap_y[s.cur]),
+                     *reinterpret_cast<const CUtensorMap*>(s.tmap_ym[s.cur]),
                      static_cast<S*>(s.buf[s.cur ^ 1]), p, make_pair_constants(p), s.derr, sc);
 }
 
@@ -540,18 +646,26 @@ cudaError_t launch_ym(Solver& s) {
 // their conversions and stochastic rounding in either kernel, on larger meshes
 // only.  us a step, tile kernel and this one: FP32 512^2 6.5 / 7.0, 900^2 15.9 /
 // 15.3, 1024^2 19.4 / 15.4, 2049^2 74 / 54, 4096^2 277 / 193; BF16 1024^2 18.2 /
-// 18.4, 1400^2 32.4 / 30.6, 4096^2 246 / 234.
+// 18.4, 1400^2 32.4 / 30.6, 4096^2 246 / 234; FP16NEQ 775^2 17.7 / 13.7, 2049^2
+// 104 / 84, 4096^2 385 / 310 (at two CTAs an SM: at three, 96 registers, it
+// spills and takes 423).
 constexpr long long kYmMinNodes = 600000, kYmMinNodes16 = 1500000;
-bool step_2d_ym_takes(int nx, int ny, int elem, size_t plane_bytes) {
+bool step_2d_ym_takes(int nx, int ny, int precision, size_t plane_bytes) {
   return nx >= 16 && ny >= 2 * kYmMinRows + 2 && plane_bytes < (size_t)1 << 31 &&
-         (long long)nx * ny >= (elem == 4 ? kYmMinNodes : kYmMinNodes16);
+         (long long)nx * ny >=
+             (precision == ISLBM_FP16DEV || precision == ISLBM_BF16DEV ? kYmMinNodes16 : kYmMinNodes);
 }
 
-// TMA box (x, y, planes) of a staged row pair.
-void step_2d_ym_box(int elem, unsigned (&box)[3]) {
-  box[0] = (unsigned)(elem == 4 ? YmGeom<float, 2>::TW : YmGeom<__half, 2>::TW);
-  box[1] = 2;
+// TMA boxes (x, y, planes) of a staged row pair: the populations, and the
+// moments of the FP16NEQ form.
+void step_2d_ym_box(int precision, unsigned (&box)[3], unsigned (&moments)[3]) {
+  box[0] = (unsigned)(precision == ISLBM_FP32      ? YmGeom<float, 2>::TW
+                      : precision == ISLBM_FP16NEQ ? YmGeom<Neq16, 2>::TW
+                                                   : YmGeom<__half, 2>::TW);
+  box[1] = moments[1] = 2;
   box[2] = 14;
+  moments[0] = (unsigned)YmGeom<Neq16, 2>::MW;
+  moments[2] = 4;
 }
 
 cudaError_t launch_step_2d_ym(Solver& s, int steps) {
@@ -561,6 +675,7 @@ cudaError_t launch_step_2d_ym(Solver& s, int steps) {
     case ISLBM_FP32: e = launch_ym<float, 2>(s); break;
     case ISLBM_FP16DEV: e = launch_ym<__half, 2>(s); break;
     case ISLBM_BF16DEV: e = launch_ym<__nv_bfloat16, 2>(s); break;
+    case ISLBM_FP16NEQ: e = launch_ym<Neq16, 2>(s); break;
   }
   if (e == cudaSuccess) s.cur ^= 1;
   return e;

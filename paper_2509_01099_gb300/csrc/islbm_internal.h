@@ -204,6 +204,7 @@ struct Solver {
   alignas(128) unsigned char tmap[2][128];   // TMA descriptors of buf[0] / buf[1]
   alignas(128) unsigned char tmap_m[2][128]; // FP16NEQ: of their moment planes
   alignas(128) unsigned char tmap_y[2][128]; // of a row pair (the 2-D marching kernel)
+  alignas(128) unsigned char tmap_ym[2][128];  // FP16NEQ: of their moments
   bool marching = false;          // 2-D: two steps in one launch where two are due
   alignas(128) unsigned char tmap3[2][7][128];   // 3-D: one descriptor per box shape
   // CUDA graphs of kGraphSteps steps, one per starting buffer, replayed on a
@@ -239,8 +240,8 @@ cudaError_t launch_reduce(Solver& s);
 cudaError_t launch_steps(Solver& s, long long want, int* done);
 // 2-D marching kernel (two steps a launch): whether it takes a mesh, its TMA box
 cudaError_t launch_step_2d_ym(Solver& s, int steps);
-bool step_2d_ym_takes(int nx, int ny, int elem, size_t plane_bytes);
-void step_2d_ym_box(int elem, unsigned (&box)[3]);
+bool step_2d_ym_takes(int nx, int ny, int precision, size_t plane_bytes);
+void step_2d_ym_box(int precision, unsigned (&box)[3], unsigned (&moments)[3]);
 
 cudaError_t launch_init_fields_3d(Solver& s, const double* rho, const double* T,
                                   const double* u0, const double* u1, const double* u2);
