@@ -1447,11 +1447,16 @@ cudaError_t launch_tma(const Solver& s, int cur, S* out, const P2<float>& p) {
   const int grid = std::min(ntiles, s.sm_count * blocks_per_sm);
   // claimed tiles pay off once a CTA walks more than a few dozen tiles
   const int k0 = tma_first_claim(ntiles, grid, STAGES);
-  // few tiles a CTA: the launch gap is a good part of the step (FP32 64 x 8
-  // tiles, 257^2 4.5 -> 4.2 us, 512^2 7.0 -> 6.5); beyond, and in the 64 x 16
-  // tiles of the 16-bit forms, early blocks cost more than they hide (BF16
-  // 1024^2 18.3 -> 21.2 us)
-  const bool serial = std::is_same<S, float>::value && R == 2 && ntiles <= 4 * grid;
+  // The next step's blocks may start early where that was measured faster (FP32
+  // 64 x 8 tiles, us a step, ordinary and early): one tile a CTA and more CTAs
+  // than SMs (257^2, 165 tiles 4.47 / 4.07, 384^2, 288 tiles 5.02 / 4.79), or a
+  // quarter of the SMs (64^2 3.50 / 3.35).  In between, a step and the next one
+  // do not both fit one block an SM (227^2, 116 tiles 3.64 / 4.14); beyond, and
+  // in the 64 x 16 tiles of the 16-bit forms, early blocks crowd on the SMs that
+  // finish first (600^2 8.32 / 8.77, BF16 1024^2 18.3 / 21.2).
+  const bool serial = std::is_same<S, float>::value && R == 2 &&
+                      (4 * ntiles <= s.sm_count ||
+                       (ntiles > s.sm_count && ntiles <= 2 * s.sm_count));
   return launch_grid(serial, k_step_tma<S, R, STAGES>, grid, kThreads, smem, s.stream,
                      *reinterpret_cast<const CUtensorMap*>(s.tmap[cur]),
                      *reinterpret_cast<const CUtensorMap*>(s.tmap_m[cur]), out, p, s.derr, k0);
