@@ -107,7 +107,8 @@ def peaks():
 
 
 KERNEL_SOURCES = {
-    2: ("islbm_d2.cu", "islbm_lanes.cuh", "islbm_store.cuh", "islbm_tma.cuh"),
+    2: ("islbm_d2.cu", "islbm_d2_common.cuh", "islbm_lanes.cuh", "islbm_store.cuh",
+        "islbm_tma.cuh"),
     3: ("islbm_d3_zm.cu", "islbm_d3_common.cuh", "islbm_lanes.cuh", "islbm_store.cuh",
         "islbm_tma.cuh"),
 }
