@@ -1466,9 +1466,9 @@ dim3 block2() { return dim3(32, 8); }
 dim3 grid2(const Solver& s) { return dim3((s.n[0] + 31) / 32, (s.n[1] + 7) / 8); }
 // Rows of a direct step's block (32 columns, one warp a row): 8, fewer where
 // that would leave SMs without a block.  A scheduler's FP64 unit takes 64 cycles
-// for a warp's instruction, so the 243 of a node's FP64 step keep it busy for
-// 7.5 us whatever the mesh: a small mesh has to spread its warps over all SMs
-// (64^2: 16 blocks of 8 warps 18.5 us a step, 128 blocks of one 11.6 us).
+// for a warp's instruction, so a mesh of few warps has to spread them over all
+// SMs (FP64, 160^2: blocks of 8 rows 18.6 us a step, of one row 15.5; from 257^2
+// on the two are the same).
 int step_block_rows(const Solver& s) {
   const long long warps = (long long)((s.n[0] + 31) / 32) * step_rows(s);
   int rows = 8;
