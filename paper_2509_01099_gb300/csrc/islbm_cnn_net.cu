@@ -97,10 +97,24 @@ __host__ __device__ constexpr int up16(int c) { return (c + 15) / 16 * 16; }
 // into different banks for every channel count in use (pitches 48 to 144 bytes)
 __host__ __device__ constexpr int pitch_of(int c) { return up16(c) + 8; }
 
+// A load of an image.  The read-only path (__ldg) is for data that nothing
+// writes while the kernel runs, and its loads are not ordered by grid_wait: not
+// for an image that the launch before may still be writing when this kernel
+// starts (LIVE), which takes ordinary loads.
+template <bool LIVE, typename V>
+__device__ __forceinline__ V load_image(const V* s) {
+  if constexpr (LIVE) {
+    return *s;
+  } else {
+    return __ldg(s);
+  }
+}
+
 // Stages the window [wy0, wy0 + rows) x [wx0, wx0 + cols) of an NHWC FP32
 // image of C channels as BF16 [pixel][pitch_of(C)]; zeros outside the image
-// and in the padding channels.
-__device__ __forceinline__ void stage_window(bf16* dst, const float* __restrict__ img, int H, int W,
+// and in the padding channels.  LIVE: see load_image.
+template <bool LIVE>
+__device__ __forceinline__ void stage_window(bf16* dst, const float* img, int H, int W,
                                              int C, int wy0, int wx0, int rows, int cols, int vec,
                                              int tid, int threads) {
   // a thread keeps its four channels and walks the pixels, four loads in flight
@@ -117,12 +131,12 @@ __device__ __forceinline__ void stage_window(bf16* dst, const float* __restrict_
       if (p + i * step < n && y >= 0 && y < H && x >= 0 && x < W) {
         const float* s = img + (y * W + x) * C + c;
         if (vec) {
-          if (c < C) v[i] = __ldg(reinterpret_cast<const float4*>(s));
+          if (c < C) v[i] = load_image<LIVE>(reinterpret_cast<const float4*>(s));
         } else {
-          if (c < C) v[i].x = __ldg(s);
-          if (c + 1 < C) v[i].y = __ldg(s + 1);
-          if (c + 2 < C) v[i].z = __ldg(s + 2);
-          if (c + 3 < C) v[i].w = __ldg(s + 3);
+          if (c < C) v[i].x = load_image<LIVE>(s);
+          if (c + 1 < C) v[i].y = load_image<LIVE>(s + 1);
+          if (c + 2 < C) v[i].z = load_image<LIVE>(s + 2);
+          if (c + 3 < C) v[i].w = load_image<LIVE>(s + 3);
         }
       }
       r += dr;
@@ -196,8 +210,8 @@ __global__ void __launch_bounds__(128) k_conv_fwd(Conv p) {
     tl.at(t, TR, b, y0, x0);
     const int wy0 = (y0 - 1) >> p.up, wx0 = (x0 - 1) >> p.up;
     __syncthreads();   // the window of the tile before is read
-    stage_window(sx, p.x + (size_t)b * Hx * Wx * p.cin, Hx, Wx, p.cin, wy0, wx0, rows, cols, p.vx,
-                 threadIdx.x, 128);
+    stage_window<true>(sx, p.x + (size_t)b * Hx * Wx * p.cin, Hx, Wx, p.cin, wy0, wx0, rows, cols,
+                       p.vx, threadIdx.x, 128);
     __syncthreads();
     float acc[MT][NT][4], tot[MT][NT][4];
 #pragma unroll
@@ -336,8 +350,8 @@ __global__ void __launch_bounds__(128) k_conv_dgrad(Conv p) {
     int b, y0, x0;
     tl.at(t, TR, b, y0, x0);
     __syncthreads();
-    stage_window(sd, p.d + (size_t)b * p.H * p.W * p.cout, p.H, p.W, p.cout, y0 - 1, x0 - 1, TR + 2,
-                 cols, p.vd, threadIdx.x, 128);
+    stage_window<false>(sd, p.d + (size_t)b * p.H * p.W * p.cout, p.H, p.W, p.cout, y0 - 1, x0 - 1,
+                        TR + 2, cols, p.vd, threadIdx.x, 128);
     __syncthreads();
     float sum[2][NT][4];
 #pragma unroll
@@ -456,8 +470,8 @@ __global__ void __launch_bounds__(512) k_conv_wgrad(Wgrad g) {
   const int nn = min(NB, p.cout - n0);
   auto stage = [&](int f, int buf, int tid, int threads) {
     const int b = f / g.phases, y0 = (f - b * g.phases) * g.pr;
-    stage_window(sx + buf * xsize, p.x + (size_t)b * Hx * Wx * p.cin, Hx, Wx, p.cin,
-                 (y0 - 1) >> p.up, -1, rows, cols, p.vx, tid, threads);
+    stage_window<false>(sx + buf * xsize, p.x + (size_t)b * Hx * Wx * p.cin, Hx, Wx, p.cin,
+                        (y0 - 1) >> p.up, -1, rows, cols, p.vx, tid, threads);
     const float* img = p.d + ((size_t)b * p.H + y0) * p.W * p.cout + n0;
     const int pixels = min(g.pr, p.H - y0) * p.W;
     bf16* dst = sd + buf * dsize;
