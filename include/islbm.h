@@ -440,8 +440,9 @@ ISLBM_API islbm_status islbm_cnn_adam(float* w, void* wb, const float* g, float*
  * call returns).  Written: zk [batch][16] (the features rounded to bf16; may be
  * NULL), h1 [batch][hidden], acts[0 .. stages]: the second layer's output and
  * every stage's.  acts 16-byte aligned.  Limits: 64 channels, 8 stages, 512
- * hidden units, 256 x 256 outputs (a wide layer fewer,
- * by its shared memory); ISLBM_ERR_ARG beyond them. */
+ * hidden units, 256 x 256 outputs (a wide layer fewer, by its shared memory),
+ * 2^30 output pixels in a batch, and fewer than 2^27 images of 1 or 2 rows (the
+ * weight gradient pads them to 16 pixels); ISLBM_ERR_ARG beyond them. */
 ISLBM_API islbm_status islbm_cnn_forward(int stages, const int* channels, int base, int hidden,
                                          const void* const* params, const float* z, int batch,
                                          float* zk, float* h1, float* const* acts, void* stream);

@@ -744,14 +744,15 @@ __global__ void __launch_bounds__(128) k_fc_fwd(Fc p, const __grid_constant__ ZA
     }
 }
 
-// dh1 = (d2 W2^T) (1 - h1^2): 16 samples and 8 hidden units a block; its 16
-// warps take chunks of `kchunk` columns, which are added in order.
+// dh1 = (d2 W2^T) (1 - h1^2): 16 samples (grid x, which takes any batch) and 8
+// hidden units (grid y) a block; its 16 warps take chunks of `kchunk` columns,
+// which are added in order.
 __global__ void __launch_bounds__(512) k_fc_dh(const float* __restrict__ d2,
                                                const bf16* __restrict__ w2,
                                                const float* __restrict__ h1, float* __restrict__ dh1,
                                                int B, int hidden, int n2, int kchunk) {
   __shared__ float part[16][kFcB * 8];
-  const int k0 = blockIdx.x * 8, bb = blockIdx.y * kFcB;
+  const int k0 = blockIdx.y * 8, bb = blockIdx.x * kFcB;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane >> 2, tig = lane & 3;
   const int chunks = (n2 + kchunk - 1) / kchunk;
   const float* r0 = d2 + (size_t)min(bb + grp, B - 1) * n2;
@@ -1037,7 +1038,7 @@ bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) &
 
 // what the fused kernels take: up to 64 channels and 8 stages, an even second
 // layer, 16-byte aligned tensors
-bool net_ok(int stages, const int* ch, int base, int hidden, int batch) {
+bool net_ok(int stages, const int* ch, int base, int hidden, int batch, int sms) {
   if (stages < 1 || stages > kMaxStages || !ch || base < 1 || hidden < 1 || hidden > kMaxHidden ||
       batch < 1)
     return false;
@@ -1050,7 +1051,10 @@ bool net_ok(int stages, const int* ch, int base, int hidden, int batch) {
   for (int s = 0; s < stages; ++s) {
     const int up = s + 1 < stages;
     if (up) H *= 2;
-    if (wgrad_plan(1, H, ch[s], ch[s + 1], up, 1).smem > (size_t)kSmemLimit) return false;
+    const WgradPlan w = wgrad_plan(batch, H, ch[s], ch[s + 1], up, sms);
+    if (w.smem > (size_t)kSmemLimit) return false;
+    // and its padded pixels a 32-bit index (images of 1 or 2 rows are padded most)
+    if ((long long)batch * w.phases * w.kp + w.kchunk > INT_MAX) return false;
   }
   return true;
 }
@@ -1099,14 +1103,14 @@ islbm_status status_of(cudaError_t e) { return e == cudaSuccess ? ISLBM_OK : ISL
 extern "C" islbm_status islbm_cnn_forward(int stages, const int* channels, int base, int hidden,
                                           const void* const* params, const float* z, int batch,
                                           float* zk, float* h1, float* const* acts, void* stream) {
-  if (!net_ok(stages, channels, base, hidden, batch) || !params || !z || !h1 || !acts)
+  const int sms = sm_count();
+  if (!net_ok(stages, channels, base, hidden, batch, sms) || !params || !z || !h1 || !acts)
     return ISLBM_ERR_ARG;
   for (int k = 0; k < 4 + 2 * stages; ++k)
     if (!params[k] || !aligned(params[k], 4)) return ISLBM_ERR_ARG;
   for (int s = 0; s <= stages; ++s)
     if (!acts[s] || !aligned(acts[s], 16)) return ISLBM_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int sms = sm_count();
   Fc f{static_cast<const bf16*>(params[0]), static_cast<const bf16*>(params[2]),
        static_cast<const float*>(params[1]), static_cast<const float*>(params[3]), zk, h1, acts[0],
        batch, hidden, base * base * channels[0], hidden % 8 == 0 && aligned(params[0], 16),
@@ -1140,8 +1144,9 @@ extern "C" islbm_status islbm_cnn_forward(int stages, const int* channels, int b
 
 extern "C" islbm_status islbm_cnn_backward_scratch(int stages, const int* channels, int base,
                                                    int hidden, int batch, unsigned long long* bytes) {
-  if (!bytes || !net_ok(stages, channels, base, hidden, batch)) return ISLBM_ERR_ARG;
-  *bytes = back_plan(stages, channels, base, hidden, batch, sm_count()).total * sizeof(float);
+  const int sms = sm_count();
+  if (!bytes || !net_ok(stages, channels, base, hidden, batch, sms)) return ISLBM_ERR_ARG;
+  *bytes = back_plan(stages, channels, base, hidden, batch, sms).total * sizeof(float);
   return ISLBM_OK;
 }
 
@@ -1150,7 +1155,8 @@ extern "C" islbm_status islbm_cnn_backward(int stages, const int* channels, int 
                                            const float* h1, const float* const* acts,
                                            const float* dy, float* const* grads, float* scratch,
                                            void* stream) {
-  if (!net_ok(stages, channels, base, hidden, batch) || !params || !zk || !h1 || !acts || !dy ||
+  const int sms = sm_count();
+  if (!net_ok(stages, channels, base, hidden, batch, sms) || !params || !zk || !h1 || !acts || !dy ||
       !grads || !scratch || !aligned(scratch, 256))
     return ISLBM_ERR_ARG;
   for (int k = 0; k < 4 + 2 * stages; ++k)
@@ -1158,7 +1164,6 @@ extern "C" islbm_status islbm_cnn_backward(int stages, const int* channels, int 
   for (int s = 0; s < stages; ++s)
     if (!acts[s] || !aligned(acts[s], 16)) return ISLBM_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int sms = sm_count();
   const BackPlan bp = back_plan(stages, channels, base, hidden, batch, sms);
   float* at = scratch;
   auto take = [&](size_t n) {
@@ -1206,7 +1211,7 @@ extern "C" islbm_status islbm_cnn_backward(int stages, const int* channels, int 
   k_bias_sum<<<sum_first, 512, 0, st>>>(sums);
   k_grad_sum<<<first, 64, 0, st>>>(segs);
   const int n2 = base * base * channels[0];
-  k_fc_dh<<<dim3((hidden + 7) / 8, (batch + kFcB - 1) / kFcB), 512, 0, st>>>(
+  k_fc_dh<<<dim3((batch + kFcB - 1) / kFcB, (hidden + 7) / 8), 512, 0, st>>>(
       d, static_cast<const bf16*>(params[2]), h1, dh1, batch, hidden, n2,
       gemm_kchunk(batch, hidden, n2, sms));
   const FcGrad l2{h1, d, grads[2], grads[3], hidden, n2, (n2 + 255) / 256, (hidden + 15) / 16};
