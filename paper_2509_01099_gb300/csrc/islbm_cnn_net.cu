@@ -625,7 +625,7 @@ struct GradSeg {
   int blocks, values, zeros, first;   // zeros: values behind them set to zero
 };
 struct GradSegs {
-  GradSeg s[2 * kMaxStages];
+  GradSeg s[2 * kMaxStages + 4];
   int n;
 };
 
@@ -793,44 +793,87 @@ __global__ void __launch_bounds__(512) k_fc_dh(const float* __restrict__ d2,
   }
 }
 
-// dW[k][n] = sum_b bf16(a[b][k]) bf16(d[b][n]) and db[n] = sum_b d[b][n] of
-// both fully connected layers in one launch: a block takes 256 columns and 16
-// rows.
+// Weight and bias gradients of both fully connected layers in one launch:
+// dW[k][n] = sum_b bf16(a[b][k]) bf16(d[b][n]) and db[n] = sum_b d[b][n], summed
+// as the chain sums them: the products in steps of 16 samples on the tensor
+// cores and, where the chain splits K, in chunks of `kchunk` samples; the biases
+// by eight interleaved lanes in chunks of kSumRows samples.  (One FP32 chain
+// over the batch, as an earlier form summed both, has 1.2 times the RMS error at
+// 16 samples and 3.8 times at 4,096.)  Chunks are blocks of their own; where
+// there are several, dw and db are their partial sums, which k_grad_sum adds.
+// A weight block takes 16 rows and 256 columns, a warp 32 of them, and reads
+// its fragments from global memory; a bias block takes 32 columns.
 struct FcGrad {
   const float *a, *d;
   float *dw, *db;
-  int K, N, gx, gy;
+  int K, N, gx, gy;              // column and row tiles
+  int kchunk, wchunks, bchunks;
+  __host__ __device__ int wblocks() const { return gx * gy * wchunks; }
+  __host__ __device__ int bblocks() const { return (N + 31) / 32 * bchunks; }
 };
+__device__ __forceinline__ void fc_weight_block(const FcGrad& p, int t, int B) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane >> 2, tig = lane & 3;
+  const int tile = t % (p.gx * p.gy), chunk = t / (p.gx * p.gy);
+  const int n0 = tile % p.gx * 256 + warp * 32, k0 = tile / p.gx * 16;
+  const int b1 = min((long long)B, (long long)(chunk + 1) * p.kchunk);
+  float acc[4][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[j][r] = 0.f;
+  // a pair of samples b, b + 1 of column c of x [B][C]
+  auto pair = [&](const float* x, int C, int b, int c) {
+    const float u = c < C && b < b1 ? __ldg(x + (size_t)b * C + c) : 0.f;
+    const float v = c < C && b + 1 < b1 ? __ldg(x + (size_t)(b + 1) * C + c) : 0.f;
+    return pack2(u, v);
+  };
+  for (int b0 = chunk * p.kchunk; b0 < b1; b0 += 16) {
+    const int b = b0 + 2 * tig;
+    const unsigned af[4] = {pair(p.a, p.K, b, k0 + grp), pair(p.a, p.K, b, k0 + grp + 8),
+                            pair(p.a, p.K, b + 8, k0 + grp), pair(p.a, p.K, b + 8, k0 + grp + 8)};
+    unsigned bf[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      bf[j][0] = pair(p.d, p.N, b, n0 + 8 * j + grp);
+      bf[j][1] = pair(p.d, p.N, b + 8, n0 + 8 * j + grp);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mma16816(acc[j], af, bf[j][0], bf[j][1]);
+  }
+  float* o = p.dw + (size_t)chunk * p.K * p.N;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int k = k0 + grp + (r >= 2 ? 8 : 0), n = n0 + 8 * j + 2 * tig + (r & 1);
+      if (k < p.K && n < p.N) o[(size_t)k * p.N + n] = acc[j][r];
+    }
+}
+__device__ __forceinline__ void fc_bias_block(const FcGrad& p, int t, int B) {
+  __shared__ float sh[8][33];
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, tiles = (p.N + 31) / 32;
+  const int chunk = t / tiles, n = t % tiles * 32 + lane;
+  const long long b1 = min((long long)B, (long long)(chunk + 1) * kSumRows);
+  float s = 0.f;
+  if (n < p.N)
+    for (long long b = (long long)chunk * kSumRows + row; b < b1; b += 8)
+      s += __ldg(p.d + (size_t)b * p.N + n);
+  sh[row][lane] = s;
+  __syncthreads();
+  if (row != 0 || n >= p.N) return;
+  float v = 0.f;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) v += sh[r][lane];
+  p.db[(size_t)chunk * p.N + n] = v;
+}
 __global__ void __launch_bounds__(256) k_fc_wgrad(FcGrad l2, FcGrad l1, int B) {
   int t = blockIdx.x;
-  const bool first = t < l2.gx * l2.gy;
-  const FcGrad p = first ? l2 : l1;
-  if (!first) t -= l2.gx * l2.gy;
-  const int n = (t % p.gx) * 256 + threadIdx.x, k0 = (t / p.gx) * 16;
-  __shared__ float sa[32][16];
-  float acc[16], db = 0.f;
-#pragma unroll
-  for (int k = 0; k < 16; ++k) acc[k] = 0.f;
-  for (int b0 = 0; b0 < B; b0 += 32) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < 32 * 16; e += 256) {
-      const int b = b0 + e / 16, k = k0 + e % 16;
-      sa[e / 16][e % 16] = b < B && k < p.K ? round_bf16(p.a[(size_t)b * p.K + k]) : 0.f;
-    }
-    __syncthreads();
-    if (n < p.N)
-      for (int b = b0; b < min(B, b0 + 32); ++b) {
-        const float v = p.d[(size_t)b * p.N + n], r = round_bf16(v);
-        db += v;
-#pragma unroll
-        for (int k = 0; k < 16; ++k) acc[k] = fmaf(sa[b - b0][k], r, acc[k]);
-      }
-  }
-  if (n >= p.N) return;
-#pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (k0 + k < p.K) p.dw[(size_t)(k0 + k) * p.N + n] = acc[k];
-  if (k0 == 0) p.db[n] = db;
+  if (t < l2.wblocks()) return fc_weight_block(l2, t, B);
+  t -= l2.wblocks();
+  if (t < l1.wblocks()) return fc_weight_block(l1, t, B);
+  t -= l1.wblocks();
+  const bool second = t < l2.bblocks();
+  fc_bias_block(second ? l2 : l1, second ? t : t - l2.bblocks(), B);
 }
 
 // Adam over all tensors of the network in one launch (the arithmetic of
@@ -904,6 +947,17 @@ int gemm_kchunk(long long M, int N, int K, int sms) {
   if (tiles < 2LL * sms && K >= 512)
     split = std::max(1, (int)std::min<long long>((2LL * sms + tiles - 1) / tiles, K / 256));
   return ((K + split - 1) / split + 63) / 64 * 64;
+}
+
+// The same for a product whose operands take the chain's tensor-core kernel
+// (tc: leading dimensions in multiples of 8, K above 32) or its mma.sync one.
+int chain_kchunk(long long M, int N, int K, bool tc, int sms) {
+  if (tc && K > 32) return gemm_kchunk(M, N, K, sms);
+  const long long tiles = (M + 63) / 64 * ((N + 63) / 64);
+  long long split = 1;
+  if (tiles < 2LL * sms && K >= 512)
+    split = std::max(1LL, std::min((2LL * sms + tiles - 1) / tiles, (long long)K / 256));
+  return (int)(((K + split - 1) / split + 31) / 32 * 32);
 }
 
 int round_nt(int n8) { return n8 <= 2 ? std::max(n8, 1) : n8 <= 4 ? 4 : n8 <= 6 ? 6 : 8; }
@@ -1006,19 +1060,9 @@ WgradPlan wgrad_plan(int B, int H, int cin, int cout, int up, int sms) {
     if (w.smem <= (size_t)kSmemLimit) break;
   }
   w.phases = (H + w.pr - 1) / w.pr;
-  // the chunks of the GEMM chain's split (gemm_kchunk; the mma.sync form where
-  // the output channels are not a multiple of 8)
+  // the chunks of the GEMM chain's split
   const long long K = (long long)B * H * H;
-  const int M = up16(9 * cin);
-  if (cout % 8 == 0) {
-    w.kchunk = gemm_kchunk(M, cout, (int)K, sms);
-  } else {
-    const long long tiles = (long long)((M + 63) / 64) * ((cout + 63) / 64);
-    long long split = 1;
-    if (tiles < 2LL * sms && K >= 512)
-      split = std::max(1LL, std::min((2LL * sms + tiles - 1) / tiles, K / 256));
-    w.kchunk = (int)(((K + split - 1) / split + 31) / 32 * 32);
-  }
+  w.kchunk = chain_kchunk(up16(9 * cin), cout, (int)K, cout % 8 == 0, sms);
   w.blocks = (int)(((long long)B * w.phases * w.kp + w.kchunk - 1) / w.kchunk);
   w.chunks = (int)((K + kSumRows - 1) / kSumRows);
   w.floats = (size_t)w.blocks * 9 * cin * cout;
@@ -1066,10 +1110,30 @@ size_t round64(size_t n) { return (n + 63) / 64 * 64; }
 struct BackPlan {
   size_t image[kMaxStages], total;
   WgradPlan w[kMaxStages];
+  FcGrad l1, l2;           // chunks and tiles; the pointers are set by the launch
 };
+// The chunks of one fully connected layer's gradients, K inputs and N outputs.
+FcGrad fc_plan(int K, int N, int batch, int sms) {
+  FcGrad g{};
+  g.K = K;
+  g.N = N;
+  g.gx = (N + 255) / 256;
+  g.gy = (K + 15) / 16;
+  g.kchunk = chain_kchunk(K, N, batch, K % 8 == 0 && N % 8 == 0, sms);
+  g.wchunks = (batch + g.kchunk - 1) / g.kchunk;
+  g.bchunks = (batch + kSumRows - 1) / kSumRows;
+  return g;
+}
+// floats of its partial sums (none where there is one chunk)
+size_t fc_floats(const FcGrad& g) {
+  return (g.wchunks > 1 ? round64((size_t)g.wchunks * g.K * g.N) : 0) +
+         (g.bchunks > 1 ? round64((size_t)g.bchunks * g.N) : 0);
+}
 BackPlan back_plan(int stages, const int* ch, int base, int hidden, int batch, int sms) {
   BackPlan b;
-  b.total = round64((size_t)batch * hidden);
+  b.l2 = fc_plan(hidden, base * base * ch[0], batch, sms);
+  b.l1 = fc_plan(kFeat, hidden, batch, sms);
+  b.total = round64((size_t)batch * hidden) + fc_floats(b.l2) + fc_floats(b.l1);
   int H = base;
   for (int s = 0; s < stages; ++s) {
     b.image[s] = round64((size_t)batch * H * H * ch[s]);
@@ -1209,14 +1273,30 @@ extern "C" islbm_status islbm_cnn_backward(int stages, const int* channels, int 
     d = c.out;
   }
   k_bias_sum<<<sum_first, 512, 0, st>>>(sums);
-  k_grad_sum<<<first, 64, 0, st>>>(segs);
   const int n2 = base * base * channels[0];
   k_fc_dh<<<dim3((batch + kFcB - 1) / kFcB, (hidden + 7) / 8), 512, 0, st>>>(
       d, static_cast<const bf16*>(params[2]), h1, dh1, batch, hidden, n2,
       gemm_kchunk(batch, hidden, n2, sms));
-  const FcGrad l2{h1, d, grads[2], grads[3], hidden, n2, (n2 + 255) / 256, (hidden + 15) / 16};
-  const FcGrad l1{zk, dh1, grads[0], grads[1], kFeat, hidden, (hidden + 255) / 256, 1};
-  k_fc_wgrad<<<l2.gx * l2.gy + l1.gx * l1.gy, 256, 0, st>>>(l2, l1, batch);
+  auto fc = [&](FcGrad g, const float* a, const float* dd, float* dw, float* db) {
+    g.a = a;
+    g.d = dd;
+    g.dw = dw;
+    g.db = db;
+    if (g.wchunks > 1) {
+      g.dw = take((size_t)g.wchunks * g.K * g.N);
+      add_seg(g.dw, dw, g.wchunks, g.K * g.N, 0);
+    }
+    if (g.bchunks > 1) {
+      g.db = take((size_t)g.bchunks * g.N);
+      add_seg(g.db, db, g.bchunks, g.N, 0);
+    }
+    return g;
+  };
+  const FcGrad l2 = fc(bp.l2, h1, d, grads[2], grads[3]);
+  const FcGrad l1 = fc(bp.l1, zk, dh1, grads[0], grads[1]);
+  k_fc_wgrad<<<l2.wblocks() + l1.wblocks() + l2.bblocks() + l1.bblocks(), 256, 0, st>>>(l2, l1,
+                                                                                       batch);
+  k_grad_sum<<<first, 64, 0, st>>>(segs);
   return status_of(cudaGetLastError());
 }
 
