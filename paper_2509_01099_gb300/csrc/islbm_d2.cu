@@ -396,11 +396,11 @@ __device__ __forceinline__ NodeState node_state_fp64(const R (&fr)[9], const R (
 }
 
 // FP32 values (every storage form but FP64) are summed on the integer units
-// (islbm_exactsum.cuh): 7 or 8 FP64 operations a node instead of about 60 with
-// the conversions and divisions.
+// (islbm_exactsum.cuh): 9 or 10 FP64 operations a node instead of about 60 with
+// the conversions and divisions, and with smaller rounding errors than those.
 template <typename S>
 __device__ __forceinline__ NodeState node_state(const S* __restrict__ s, size_t idx,
-                                                long long P, float aT, double gbeta, double Ts,
+                                                long long P, float aT, Force force, double Ts,
                                                 double Tref) {
   using R = typename Store<S>::R;
   R f[9], g[5];
@@ -414,30 +414,31 @@ __device__ __forceinline__ NodeState node_state(const S* __restrict__ s, size_t 
     for (int i = 0; i < 5; ++i) G += aligned(g[i], Eg);
     const long long ax = F[1] + F[3], ay = F[2] + F[4];
     const long long dp = F[5] - F[7], dm = F[6] - F[8], pp = F[5] + F[7], pm = F[6] + F[8];
-    NodeState n;
-    n.rho = 1.0 + aligned_to_double(F[0] + ax + ay + pp + pm, Ef);
-    if (max(Ef, Eg) < 255 && mid_range(n.rho)) {
+    const double d = aligned_to_double(F[0] + ax + ay + pp + pm, Ef);
+    if (max(Ef, Eg) < 255 && below_half(d)) {
       const double jx = aligned_to_double(F[1] - F[3] + dp - dm, Ef);
       const double jy = aligned_to_double(F[2] - F[4] + dp + dm, Ef);
-      const double r = quick_rcp(n.rho), h = 0.5 * gbeta;
+      const Reciprocal r(d);
+      NodeState n;
+      n.rho = 1.0 + d;
       n.T = aligned_to_double(G, Eg);
-      if (Ts != 0.0) n.T += Ts;
-      n.ux = jx * r;
-      n.uy = fma(jy, r, fma(-h, n.T, h * Tref));
+      if (force.shift) n.T += Ts;
+      n.ux = r.quotient(jx);
+      n.uy = r.quotient(jy, force.c * (n.T - Tref));
       return n;
     }
   }
-  return node_state_fp64(f, g, gbeta, Ts, Tref);
+  return node_state_fp64(f, g, force.gbeta, Ts, Tref);
 }
 
 // ACC: add the fields to the arrays (time averages) instead of writing them.
 template <typename S, bool ACC>
-__global__ void k_fields(const S* __restrict__ s, P2<typename Store<S>::R> p, double gbeta,
+__global__ void k_fields(const S* __restrict__ s, P2<typename Store<S>::R> p, Force force,
                          double Ts, double Tref, double* rho, double* T, double* u, double* v) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= p.nx || y >= p.ny) return;
-  const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, gbeta, Ts,
+  const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, force, Ts,
                                  Tref);
   const size_t node = (size_t)y * p.nx + x;
   if (rho) put_field<ACC>(rho + node, n.rho);
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(kRedThreads, 2)
 // (have_snap = 0) the old values count as zero and the buffer is only written.
 template <typename S>
 __global__ void __launch_bounds__(kRedThreads, 2)
-    k_steady(const S* __restrict__ s, P2<typename Store<S>::R> p, RowStrips tk, double gbeta,
+    k_steady(const S* __restrict__ s, P2<typename Store<S>::R> p, RowStrips tk, Force force,
              double Ts, double T0, double dT, int have_snap, double* snap, double* partial,
              double* out, int* words) {
   __shared__ double sh[kRedWarps][RED_STRIDE];
@@ -597,7 +598,7 @@ __global__ void __launch_bounds__(kRedThreads, 2)
     const int ya = strip * tk.per, yb = min(ya + tk.per, tk.rows);
     for (int y = ya; y < yb; ++y) {
       const size_t k = (size_t)y * p.nx + x;
-      const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, gbeta,
+      const NodeState n = node_state(s, (size_t)y * p.pitch + x, p.plane, (float)p.a_T, force,
                                      Ts, T0);
       const double Tn = dT == 1.0 ? n.T - T0 : (n.T - T0) / dT;
       double ou = 0.0, ov = 0.0, oT = 0.0;
@@ -1568,7 +1569,7 @@ struct FieldsFn {
     using R = typename Store<S>::R;
     const auto k = acc ? k_fields<S, true> : k_fields<S, false>;
     k<<<grid2(s), block2(), 0, s.stream>>>(static_cast<const S*>(s.buf[s.cur]), make_params<R>(s),
-                                           s.ph.gbeta, s.ph.Ts, s.ph.T0, rho, T, u, v);
+                                           make_force(s), s.ph.Ts, s.ph.T0, rho, T, u, v);
     return cudaGetLastError();
   }
 };
@@ -1601,7 +1602,7 @@ struct SteadyFn {
     using R = typename Store<S>::R;
     const RowStrips tk = row_strips(s.n[0], s.n[1], s.red_blocks);
     k_steady<S><<<tk.blocks, kRedThreads, 0, s.stream>>>(
-        static_cast<const S*>(s.buf[s.cur]), make_params<R>(s), tk, s.ph.gbeta, s.ph.Ts, s.ph.T0,
+        static_cast<const S*>(s.buf[s.cur]), make_params<R>(s), tk, make_force(s), s.ph.Ts, s.ph.T0,
         s.ph.dT, s.snap_valid ? 1 : 0, s.dsnap, s.dscratch, s.hresult, s.derr);
     return cudaGetLastError();
   }

@@ -223,7 +223,7 @@ __device__ __forceinline__ void sums3(const V (&f)[19], const V (&g)[7], V& drho
 // As the 2-D node_state: FP32 values are summed on the integer units.
 template <typename S>
 __device__ __forceinline__ NodeState3 node_state3(const S* __restrict__ s, size_t idx,
-                                                  long long P, double gbeta, double Ts,
+                                                  long long P, Force force, double Ts,
                                                   double Tref) {
   using R = typename Store<S>::R;
   R fr[19], gr[7];
@@ -240,14 +240,15 @@ __device__ __forceinline__ NodeState3 node_state3(const S* __restrict__ s, size_
 #pragma unroll
     for (int i = 0; i < 7; ++i) G[i] = aligned(gr[i], Eg);
     sums3(F, G, M, X, Y, Z, Q);
-    n.rho = 1.0 + aligned_to_double(M, Ef);
-    if (max(Ef, Eg) < 255 && mid_range(n.rho)) {
-      const double r = quick_rcp(n.rho), h = 0.5 * gbeta;
+    const double d = aligned_to_double(M, Ef);
+    if (max(Ef, Eg) < 255 && below_half(d)) {
+      const Reciprocal r(d);
+      n.rho = 1.0 + d;
       n.T = aligned_to_double(Q, Eg);
-      if (Ts != 0.0) n.T += Ts;
-      n.ux = aligned_to_double(X, Ef) * r;
-      n.uy = fma(aligned_to_double(Y, Ef), r, fma(-h, n.T, h * Tref));
-      n.uz = aligned_to_double(Z, Ef) * r;
+      if (force.shift) n.T += Ts;
+      n.ux = r.quotient(aligned_to_double(X, Ef));
+      n.uy = r.quotient(aligned_to_double(Y, Ef), force.c * (n.T - Tref));
+      n.uz = r.quotient(aligned_to_double(Z, Ef));
       return n;
     }
   }
@@ -259,7 +260,7 @@ __device__ __forceinline__ NodeState3 node_state3(const S* __restrict__ s, size_
   sums3(f, g, drho, jx, jy, jz, Tr);
   n.rho = 1.0 + drho;
   n.T = Tr + Ts;
-  const double Fy = n.rho * gbeta * (n.T - Tref);
+  const double Fy = n.rho * force.gbeta * (n.T - Tref);
   n.ux = jx / n.rho;
   n.uy = (jy - 0.5 * Fy) / n.rho;
   n.uz = jz / n.rho;
@@ -268,7 +269,7 @@ __device__ __forceinline__ NodeState3 node_state3(const S* __restrict__ s, size_
 
 // ACC: add the fields to the arrays (time averages) instead of writing them.
 template <typename S, bool ACC>
-__global__ void k_fields3(const S* __restrict__ s, P3<typename Store<S>::R> p, double gbeta,
+__global__ void k_fields3(const S* __restrict__ s, P3<typename Store<S>::R> p, Force force,
                           double Ts, double Tref, double* rho, double* T, double* u, double* v,
                           double* w) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -276,7 +277,7 @@ __global__ void k_fields3(const S* __restrict__ s, P3<typename Store<S>::R> p, d
   const int z = blockIdx.z;
   if (x >= p.nx || y >= p.ny) return;
   const NodeState3 n =
-      node_state3(s, ((size_t)z * p.ny + y) * p.pitch + x, p.plane, gbeta, Ts, Tref);
+      node_state3(s, ((size_t)z * p.ny + y) * p.pitch + x, p.plane, force, Ts, Tref);
   const size_t node = ((size_t)z * p.ny + y) * p.nx + x;
   if (rho) put_field<ACC>(rho + node, n.rho);
   if (T) put_field<ACC>(T + node, n.T);
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(kRedThreads, 2)
 // Steady-state criterion (Sec. 3) in 3-D, as the 2-D kernel with (u, v, w, T*).
 template <typename S>
 __global__ void __launch_bounds__(kRedThreads, 2)
-    k_steady3(const S* __restrict__ s, P3<typename Store<S>::R> p, RowStrips tk, double gbeta,
+    k_steady3(const S* __restrict__ s, P3<typename Store<S>::R> p, RowStrips tk, Force force,
               double Ts, double T0, double dT, int have_snap, double* snap, double* partial,
               double* out, int* words) {
   __shared__ double sh[kRedWarps][RED_STRIDE];
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(kRedThreads, 2)
     const int ra = strip * tk.per, rb = min(ra + tk.per, tk.rows);
     for (int row = ra; row < rb; ++row) {
       const size_t k = (size_t)row * p.nx + x;
-      const NodeState3 n = node_state3(s, (size_t)row * p.pitch + x, p.plane, gbeta, Ts, T0);
+      const NodeState3 n = node_state3(s, (size_t)row * p.pitch + x, p.plane, force, Ts, T0);
       const double Tn = dT == 1.0 ? n.T - T0 : (n.T - T0) / dT;
       double ou = 0.0, ov = 0.0, ow = 0.0, oT = 0.0;
       if (have_snap) {
@@ -507,7 +508,7 @@ struct Fields3 {
     using R = typename Store<S>::R;
     const auto k = acc ? k_fields3<S, true> : k_fields3<S, false>;
     k<<<grid3(s), block3(), 0, s.stream>>>(static_cast<const S*>(s.buf[s.cur]),
-                                           make_params3<R>(s), s.ph.gbeta, s.ph.Ts, s.ph.T0, rho,
+                                           make_params3<R>(s), make_force(s), s.ph.Ts, s.ph.T0, rho,
                                            T, u, v, w);
     return cudaGetLastError();
   }
@@ -541,7 +542,7 @@ struct Steady3 {
     using R = typename Store<S>::R;
     const RowStrips tk = row_strips(s.n[0], (long long)s.n[1] * s.n[2], s.red_blocks);
     k_steady3<S><<<tk.blocks, kRedThreads, 0, s.stream>>>(
-        static_cast<const S*>(s.buf[s.cur]), make_params3<R>(s), tk, s.ph.gbeta, s.ph.Ts, s.ph.T0,
+        static_cast<const S*>(s.buf[s.cur]), make_params3<R>(s), tk, make_force(s), s.ph.Ts, s.ph.T0,
         s.ph.dT, s.snap_valid ? 1 : 0, s.dsnap, s.dscratch, s.hresult, s.derr);
     return cudaGetLastError();
   }

@@ -61,28 +61,59 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
 }
 
-// Whether a is a positive normal value between 2^-60 and 2^60.
-__device__ __forceinline__ bool mid_range(double a) {
-  return ((unsigned)__double2hiint(a) >> 20) - (1023u - 60u) <= 120u;
+// FP64 value of an FP32 value that is normal or zero.
+__device__ __forceinline__ double widen_signed(float f) {
+  const unsigned b = __float_as_uint(f);
+  const unsigned hi = (b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20));
+  return f == 0.f ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
 }
 
-// 1 / a within one ulp for a value of mid_range: the FP32 reciprocal (relative
-// error below 2^-21) and one third-order correction, 3 FP64 operations.
-__device__ __forceinline__ double quick_rcp(double a) {
-  const double r = widen(__fdividef(1.0f, trunc_to_float(a)));
-  const double x = fma(-a, r, 1.0);
-  return fma(r, fma(x, x, x), r);
+// Whether |d| < 1/2 (not so for a NaN).
+__device__ __forceinline__ bool below_half(double d) {
+  return ((unsigned)__double2hiint(d) & 0x7FFFFFFFu) < 0x3FE00000u;
 }
 
-// sqrt(a) within one ulp for a = 0 and 2^-100 .. 2^100 (5 FP64 operations);
-// elsewhere the library's.
+// FP32 value of |d| < 2, truncated; 0 below 2^-30.
+__device__ __forceinline__ float trunc_small(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), m = hi & 0x7FFFFFFFu;
+  const unsigned b = ((m - (896u << 20)) << 3) | ((unsigned)__double2loint(d) >> 29);
+  return m < ((1023u - 30u) << 20) ? 0.f : __uint_as_float(b | (hi & 0x80000000u));
+}
+
+// 1 / (1 + d) = hi + lo for |d| < 1/2: hi the FP32 reciprocal (relative error below
+// 2^-21; 1 - hi is exact), x = 1 - (1 + d) hi, lo = hi (x + x^2 + ...).  Divided by
+// 1 + d, j is quotient(j): one rounding, and 2^-74 |j| from the small terms.  RMS
+// error of a component over |d| < 1/200 in units of 2^-53: 0.43, as a division
+// where 1 + d is exact (0.63 where it is rounded; the product with a rounded
+// reciprocal 0.78).  3 FP64 operations, and 2 for a quotient.
+struct Reciprocal {
+  double hi, lo;
+  __device__ __forceinline__ explicit Reciprocal(double d) {
+    const float rf = __fdividef(1.0f, 1.0f + trunc_small(d));
+    hi = widen(rf);
+    const double x = fma(-d, hi, widen_signed(1.0f - rf));
+    lo = hi * fma(x, x, x);
+  }
+  // j / (1 + d), and with c (small beside it) added before it is rounded
+  __device__ __forceinline__ double quotient(double j) const { return fma(j, hi, j * lo); }
+  __device__ __forceinline__ double quotient(double j, double c) const {
+    return fma(j, hi, fma(j, lo, c));
+  }
+};
+
+// sqrt(a) for a = 0 and 2^-100 .. 2^100, elsewhere the library's.  g = a y with
+// the FP32 reciprocal root y (relative error e below 2^-20) and two Newton steps
+// on the residual a - g^2, whose errors are 3/2 e^2 and below 2^-60: the result
+// is the correctly rounded one but for some 10^-6 of the arguments.  5 FP64
+// operations.
 __device__ __forceinline__ double quick_sqrt(double a) {
   const unsigned e = ((unsigned)__double2hiint(a) >> 20);
   if (e - (1023u - 100u) > 200u) return sqrt(a);
-  const double y = widen(rsqrtf(trunc_to_float(a)));
-  const double g = a * y;                    // sqrt(a) = g (1 - x)^(-1/2),
-  const double x = fma(-g, y, 1.0);          // x = 1 - a y^2, below 2^-20
-  return fma(g, x * fma(x, 0.375, 0.5), g);
+  const float yf = rsqrtf(trunc_to_float(a));
+  const double y = widen(yf), h = widen(0.5f * yf);
+  const double g = a * y;
+  const double s = fma(fma(-g, g, a), h, g);
+  return fma(fma(-s, s, a), h, s);
 }
 
 }  // namespace islbm

@@ -97,6 +97,16 @@ __device__ __forceinline__ void reduce_finish(const double (*sh)[RED_STRIDE], in
   }
 }
 
+// Constants of the velocities, formed on the host: an operation, or a comparison,
+// on the FP64 pipe costs the field output of 1025^2 nodes 2 us.
+struct Force {
+  double gbeta, c;   // g beta, -g beta / 2
+  int shift;         // whether T_s != 0
+};
+inline Force make_force(const Solver& s) {
+  return Force{s.ph.gbeta, -0.5 * s.ph.gbeta, s.ph.Ts != 0.0 ? 1 : 0};
+}
+
 // Adds v to *p (time averages) or writes it.
 template <bool ACC>
 __device__ __forceinline__ void put_field(double* p, double v) {
