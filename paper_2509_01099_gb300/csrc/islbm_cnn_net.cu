@@ -771,28 +771,30 @@ __global__ void __launch_bounds__(128) k_fc_fwd(Fc p, const __grid_constant__ Z 
   }
 }
 
-// dh1 = (d2 W2^T) (1 - h1^2): 16 samples (grid x, which takes any batch) and 8
-// hidden units (grid y) a block; its 16 warps take chunks of `kchunk` columns,
-// which are added in order.
+// dh1 = (d2 W2^T) (1 - h1^2).  `share` of a block's 16 warps take the chunks of
+// `kchunk` columns of one tile of 16 samples (grid x, which takes any batch) and 8
+// hidden units (grid y), which are added in order; the block's 16 / share tiles
+// are of the same samples.
 __global__ void __launch_bounds__(512) k_fc_dh(const float* __restrict__ d2,
                                                const bf16* __restrict__ w2,
                                                const float* __restrict__ h1, float* __restrict__ dh1,
-                                               int B, int hidden, int n2, int kchunk) {
+                                               int B, int hidden, int n2, int kchunk, int share) {
   __shared__ float part[16][kFcB * 8];
-  const int k0 = blockIdx.y * 8, bb = blockIdx.x * kFcB;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane >> 2, tig = lane & 3;
+  const int kb = blockIdx.y * (16 / share) * 8, bb = blockIdx.x * kFcB;
+  const int k0 = kb + warp / share * 8, mine = warp % share;
   const int chunks = (n2 + kchunk - 1) / kchunk;
   const float* r0 = d2 + (size_t)min(bb + grp, B - 1) * n2;
   const float* r1 = d2 + (size_t)min(bb + grp + 8, B - 1) * n2;
   const bf16* wr = w2 + (size_t)min(k0 + grp, hidden - 1) * n2;
-  float total = 0.f;
-  for (int c0 = 0; c0 < chunks; c0 += 16) {
-    const int nc = min(16, chunks - c0);
-    if (warp < nc) {
+  float total[4] = {0.f, 0.f, 0.f, 0.f};   // of the values threadIdx.x + 512 i of the block's tiles
+  for (int c0 = 0; c0 < chunks; c0 += share) {
+    const int nc = min(share, chunks - c0);
+    if (mine < nc && k0 < hidden) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const int e = min(n2, (c0 + warp + 1) * kchunk);
+      const int e = min(n2, (c0 + mine + 1) * kchunk);
 #pragma unroll 4
-      for (int n = (c0 + warp) * kchunk; n < e; n += 16) {
+      for (int n = (c0 + mine) * kchunk; n < e; n += 16) {
         const int c = n + 2 * tig;               // n2 is even: pairs are whole
         const bool in0 = c < e, in1 = c + 8 < e;
         auto pair = [&](const float* r, int at, bool in) {
@@ -809,14 +811,22 @@ __global__ void __launch_bounds__(512) k_fc_dh(const float* __restrict__ d2,
         part[warp][(grp + (r >= 2 ? 8 : 0)) * 8 + 2 * tig + (r & 1)] = acc[r];
     }
     __syncthreads();
-    if (threadIdx.x < kFcB * 8)
-      for (int c = 0; c < nc; ++c) total += part[c][threadIdx.x];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int v = threadIdx.x + 512 * i, tile = v / (kFcB * 8);
+      if (tile < 16 / share && kb + tile * 8 < hidden)
+        for (int c = 0; c < nc; ++c) total[i] += part[tile * share + c][v % (kFcB * 8)];
+    }
     __syncthreads();
   }
-  const int b = bb + threadIdx.x / 8, k = k0 + threadIdx.x % 8;
-  if (threadIdx.x < kFcB * 8 && b < B && k < hidden) {
-    const float h = h1[(size_t)b * hidden + k];
-    dh1[(size_t)b * hidden + k] = total * (1.f - h * h);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int v = threadIdx.x + 512 * i, tile = v / (kFcB * 8);
+    const int b = bb + v % (kFcB * 8) / 8, k = kb + tile * 8 + v % 8;
+    if (tile < 16 / share && b < B && k < hidden) {
+      const float h = h1[(size_t)b * hidden + k];
+      dh1[(size_t)b * hidden + k] = total[i] * (1.f - h * h);
+    }
   }
 }
 
@@ -1333,9 +1343,19 @@ extern "C" islbm_status islbm_cnn_backward(int stages, const int* channels, int 
   }
   k_bias_sum<<<sum_first, 512, 0, st>>>(sums);
   const int n2 = base * base * channels[0];
-  k_fc_dh<<<dim3((batch + kFcB - 1) / kFcB, (hidden + 7) / 8), 512, 0, st>>>(
-      d, static_cast<const bf16*>(params[2]), h1, dh1, batch, hidden, n2,
-      gemm_kchunk(batch, hidden, n2, sms));
+  const int dh_chunk = gemm_kchunk(batch, hidden, n2, sms), dh_tiles = (hidden + 7) / 8;
+  const int dh_x = (batch + kFcB - 1) / kFcB;
+  // Warps of a tile: all 16 of a block, half of them at a time where there are
+  // not as many chunks and the blocks still fill the GPU (a batch that fills it
+  // by itself has one chunk, and 15 warps would be idle: the backward pass of 512
+  // hidden units, 4,096 outputs and one convolution took 3.19 ms for 4,096 samples
+  // and takes 1.37, for 16,384 36.0 and 5.3).
+  int share = 16;
+  while (share > 1 && share / 2 >= (n2 + dh_chunk - 1) / dh_chunk &&
+         (long long)dh_x * dh_tiles * (share / 2) / 16 >= 2LL * sms)
+    share /= 2;
+  k_fc_dh<<<dim3(dh_x, (dh_tiles + 16 / share - 1) / (16 / share)), 512, 0, st>>>(
+      d, static_cast<const bf16*>(params[2]), h1, dh1, batch, hidden, n2, dh_chunk, share);
   auto fc = [&](FcGrad g, const float* a, const float* dd, float* dw, float* db) {
     g.a = a;
     g.d = dd;
