@@ -124,8 +124,19 @@ class WarmStartNet:
     # ---- forward ----
     def forward(self, z: np.ndarray, keep=True):
         """z: [B, 16] features.  Returns the output [B, S, S, 3] (torch, FP32)."""
-        if not (self.fused and z.shape[1] == FEATURES and 1 <= z.shape[0] <= (1 << 30) // self.size ** 2):
-            return self._forward_chain(z, keep)
+        B, pixels = z.shape[0], self.size ** 2
+        fused = self.fused and z.shape[1] == FEATURES and 1 <= B <= (1 << 30) // pixels
+        # Large batches of images of one or two rows: the fused layers' tiles of 8 x 16
+        # pixels are nearly all padding there.  Forward and backward over the chain's,
+        # networks of 1 to 2 rows and 16 or 64 channels: 4,096 samples 0.66-0.90, 16,384
+        # 1.01-1.72, 65,536 1.21-2.73 (3 rows 0.65-0.76, 0.79-0.90, 0.96-1.08).  The
+        # chain's grids end at 65,535 blocks of 64 pixels.
+        if fused and pixels <= 4 and 8192 < B <= 65535 * 64 // pixels:
+            fused = False
+        return self._forward_fused(z, keep) if fused else self._forward_chain(z, keep)
+
+    def _forward_fused(self, z, keep):
+        """forward() as fused layers, within the limits of islbm_cnn_forward."""
         B = z.shape[0]
         z = np.ascontiguousarray(z, dtype=np.float32)
         at, total = self._layout(B)

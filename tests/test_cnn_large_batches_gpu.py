@@ -71,3 +71,14 @@ def test_a_small_network_at_large_batches_is_no_slower_than_the_chain(batch):
         return min(t)
 
     assert best(lambda: net.forward(z)) <= 1.5 * best(lambda: net._forward_chain(z, True))
+
+
+@pytest.mark.parametrize("base,channels,batch,fused", [
+    (1, (16,), 8192, True), (1, (16,), 8193, False), (2, (64,), 16384, False),
+    (1, (16, 16), 20000, False), (2, (16, 16), 20000, True), (3, (16,), 20000, True),
+    (1, (2,), 65535 * 64 + 1, True),        # beyond the chain's grids
+])
+def test_tiny_images_in_large_batches_take_the_chain(base, channels, batch, fused):
+    net = _net(base=base, channels=channels, hidden=16)
+    net.forward(_z(batch))
+    assert ("flat" in net.cache) == fused
