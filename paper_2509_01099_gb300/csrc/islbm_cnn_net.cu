@@ -681,6 +681,7 @@ struct Fc {
   const float *b1, *b2;
   float *zk, *h1, *x0;           // zk may be null
   int B, hidden, n2, v1, v2;     // v1, v2: 16-byte loads of w1 and w2
+  int kchunk;                    // hidden units summed together (see gemm_kchunk)
 };
 
 // rows x cols values at src (row pitch ld), BF16, into dst (row pitch dp); zeros
@@ -751,8 +752,22 @@ __global__ void __launch_bounds__(128) k_fc_fwd(Fc p, const __grid_constant__ Z 
       }
     }
     __syncthreads();
-    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-    for (int k = 0; k < HP; k += 16) {
+    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, tot[2][4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) tot[j][r] = 0.f;
+    for (int k = 0, left = p.kchunk; k < HP; k += 16, left -= 16) {
+      if (left == 0) {
+        left = p.kchunk;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            tot[j][r] += acc[j][r];
+            acc[j][r] = 0.f;
+          }
+      }
       unsigned af[4], bq[4];
       ldsm4(af, sptr(sh) + 2u * (unsigned)((lane & 15) * P + k + (lane >> 4) * 8));
       ldsm4t(bq, sptr(sw2) + 2u * (unsigned)((k + (lane & 15)) * 72 + warp * 16 + (lane >> 4) * 8));
@@ -764,7 +779,8 @@ __global__ void __launch_bounds__(128) k_fc_fwd(Fc p, const __grid_constant__ Z 
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int b = grp + (r >= 2 ? 8 : 0), n = n0 + warp * 16 + 8 * j + 2 * tig + (r & 1);
-        if (b < nb && n < p.n2) p.x0[(size_t)(bb + b) * p.n2 + n] = tanhf(acc[j][r] + p.b2[n]);
+        if (b < nb && n < p.n2) p.x0[(size_t)(bb + b) * p.n2 + n] =
+              tanhf(tot[j][r] + acc[j][r] + p.b2[n]);
       }
     // (the next tile's features go to sz, read before the last barrier, and its
     // hidden layer to sh, behind the next one)
@@ -1257,7 +1273,9 @@ extern "C" islbm_status islbm_cnn_forward(int stages, const int* channels, int b
   Fc f{static_cast<const bf16*>(params[0]), static_cast<const bf16*>(params[2]),
        static_cast<const float*>(params[1]), static_cast<const float*>(params[3]), zk, h1, acts[0],
        batch, hidden, base * base * channels[0], hidden % 8 == 0 && aligned(params[0], 16),
-       base * base * channels[0] % 8 == 0 && aligned(params[2], 16)};
+       base * base * channels[0] % 8 == 0 && aligned(params[2], 16),
+       chain_kchunk(batch, base * base * channels[0], hidden,
+                    hidden % 8 == 0 && base * base * channels[0] % 8 == 0, sms)};
   cudaError_t e = fc_forward(f, z, sms, st);
   if (e != cudaSuccess) return status_of(e);
   int H = base;
