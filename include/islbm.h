@@ -131,7 +131,9 @@ typedef struct {
   double steps_per_tf;   /* time steps per free-fall time, L/u_f (Sec. 3)       */
   double bytes_per_update; /* algorithmic HBM bytes of one node update          */
   long long time;     /* steps taken since the last set_* call                  */
-  int kernel;         /* step-kernel variant in use (see islbm_params.kernel)    */
+  int kernel;         /* step-kernel variant of single steps (see
+                         islbm_params.kernel; with kernel = 0 a large 2-D mesh
+                         takes its steps in pairs, two in one launch)            */
   int sm_count;       /* streaming multiprocessors of the device                */
 } islbm_info_t;
 
@@ -305,7 +307,9 @@ typedef struct islbm_batch* islbm_batch_t;
 /* Time the 2-D step-kernel variants (islbm_params.kernel 1..6) of one square mesh
  * with CUDA events on `stream` (30 steps after 5 warm-up steps each) and
  * return the fastest in *best; us_per_step (host, may be NULL) receives
- * ISLBM_KERNEL_VARIANTS entries (+inf for variants that cannot run).  Results
+ * ISLBM_KERNEL_VARIANTS entries (+inf for variants that cannot run).  Entry 0
+ * (the library's choice) is timed where that advances two steps a launch, which
+ * no named variant does, and is +inf where it is one of the others.  Results
  * are cached per (n, mesh, a, precision) for the life of the process.
  * FP32 / FP16DEV / BF16DEV / FP16NEQ (which runs variants 4 and 5 only). */
 #define ISLBM_KERNEL_VARIANTS 10
@@ -315,8 +319,9 @@ ISLBM_API islbm_status islbm_autotune(int n, int mesh, double a, int precision, 
 /* Create a batch of `count` cavities (host array, copied) with one storage
  * precision (FP32 / FP16DEV / BF16DEV / FP16NEQ).  opt: common parameters
  * (NULL = defaults).  autotune != 0 chooses each mesh size's tile height with
- * islbm_autotune (FP16NEQ: always 8 rows); otherwise 8-row tiles.  stream:
- * shared by all members. */
+ * islbm_autotune (FP16NEQ: always 8 rows); otherwise 8-row tiles.  (The tiles are
+ * those of single steps: an FP32 batch that takes two steps a launch takes only a
+ * left-over one with them.)  stream: shared by all members. */
 ISLBM_API islbm_status islbm_batch_create(int count, const islbm_cavity* cavities, int precision,
                                           const islbm_params* opt, int autotune, void* stream,
                                           islbm_batch_t* out);

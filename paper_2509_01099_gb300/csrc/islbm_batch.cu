@@ -211,7 +211,7 @@ extern "C" islbm_status islbm_autotune(int n, int mesh, double a, int precision,
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
       return bfail(nullptr, ISLBM_ERR_CUDA, "islbm_autotune: events");
-    for (int k = KV_DIRECT; k < KV_COUNT; ++k) {
+    for (int k = KV_AUTO; k < KV_COUNT; ++k) {
       islbm_params prm;
       islbm_default_params(&prm);
       prm.kernel = k;
@@ -219,6 +219,10 @@ extern "C" islbm_status islbm_autotune(int n, int mesh, double a, int precision,
       if (islbm_create(xi.data(), n, xi.data(), n, nullptr, 0, 1e7, 0.71, ISLBM_D2Q9_D2Q5,
                        precision, &prm, stream, &h) != ISLBM_OK)
         continue;
+      if (k == KV_AUTO && !h->marching) {   // one of the named variants
+        islbm_destroy(h);
+        continue;
+      }
       h->use_graphs = false;
       const int warm = 5, runs = 30;
       bool ok = islbm_step(h, warm) == ISLBM_OK;
@@ -237,7 +241,7 @@ extern "C" islbm_status islbm_autotune(int n, int mesh, double a, int precision,
     g_tune_cache[key] = times;
   }
   int k_best = KV_DIRECT;
-  for (int k = KV_DIRECT; k < KV_COUNT; ++k)
+  for (int k = KV_AUTO; k < KV_COUNT; ++k)
     if (times[k] < times[k_best]) k_best = k;
   *best = k_best;
   if (us_per_step)

@@ -631,7 +631,8 @@ def islbm_reduce_noalloc(f, g, nx, ny, xi_x, xi_y, Ra, Pr=0.71, params: Params |
 
 
 def islbm_autotune(n, mesh="tanh", a=1.5, precision="fp32", stream=None):
-    """Fastest step-kernel variant of a square mesh and the per-variant step times (us)."""
+    """Fastest step-kernel variant of a square mesh (0: the library's choice, where that
+    takes two steps a launch) and the per-variant step times (us)."""
     best = ctypes.c_int()
     us = (ctypes.c_double * KERNEL_VARIANTS)()
     if stream is None:
