@@ -641,19 +641,43 @@ cudaError_t launch_ym(Solver& s) {
 }  // namespace
 
 // Whether the marching kernel takes a mesh (at least two chunks of the shortest
-// length, 32-bit offsets in a plane), and whether it is the faster one there: it
-// is once its CTAs fill the GPU, and in the 16-bit forms, which are bound by
+// length, 32-bit offsets in a plane), and whether it is the faster one there.
+//
+// It is once its CTAs fill the GPU, and in the 16-bit forms, which are bound by
 // their conversions and stochastic rounding in either kernel, on larger meshes
 // only.  us a step, tile kernel and this one: FP32 512^2 6.5 / 7.0, 900^2 15.9 /
 // 15.3, 1024^2 19.4 / 15.4, 2049^2 74 / 54, 4096^2 277 / 193; BF16 1024^2 18.2 /
 // 18.4, 1400^2 32.4 / 30.6, 4096^2 246 / 234; FP16NEQ 775^2 17.7 / 13.7, 2049^2
 // 104 / 84, 4096^2 385 / 310 (at two CTAs an SM: at three, 96 registers, it
 // spills and takes 423).
+//
+// And its strips have to be about as full as the tile kernel's tiles: a strip is
+// 62 columns (FP16NEQ 60), a tile 64, so a mesh 64 columns wide takes two half
+// empty strips for one full tile.  With f, the columns of the strips over those
+// of the tiles, measured time over the tile kernel's (columns x rows so that the
+// nodes are as given):
+//   FP32, 0.6M nodes: f = 0.97 (62, 124, 240 columns) 0.87-0.88, 1.09 (512) 0.92,
+//     1.16 (320) 1.02, 1.29 (192) 1.11, 1.45 (128) 1.17, 1.94 (64) 1.35; from
+//     1.2M on, where the tile kernel's two buffers leave L2: 1.16 0.69-0.85, 1.29
+//     0.75-0.93, 1.45 0.93-1.04, 1.94 1.06-1.19
+//   FP16NEQ: f = 0.94 0.75, 1.17 (256) 0.92-0.97, 1.25 (192) 0.97-1.02, 1.41 (128)
+//     1.08-1.15, 1.88 (64) 1.40-1.49
+//   FP16 / BF16 from 1.5M: f = 0.97 0.95, 1.03 (1024) 0.94-0.99, 1.05 (768)
+//     0.96-1.02, 1.09 (512) 0.97-1.05, 1.16 1.04-1.12, 1.45 1.28-1.37, 1.94 1.47-1.58
+// Up to 32 columns, one of a group's two warps computes nothing that is kept:
+// FP16NEQ 0.98-1.05, FP16 1.11-1.20, BF16 1.02-1.06 (FP32 0.73-0.88).
 constexpr long long kYmMinNodes = 600000, kYmMinNodes16 = 1500000;
+constexpr long long kYmL2Nodes = 1100000;   // FP32: 2 x 56 bytes of these are the L2 cache
 bool step_2d_ym_takes(int nx, int ny, int precision, size_t plane_bytes) {
-  return nx >= 16 && ny >= 2 * kYmMinRows + 2 && plane_bytes < (size_t)1 << 31 &&
-         (long long)nx * ny >=
-             (precision == ISLBM_FP16DEV || precision == ISLBM_BF16DEV ? kYmMinNodes16 : kYmMinNodes);
+  if (nx < 16 || ny < 2 * kYmMinRows + 2 || plane_bytes >= (size_t)1 << 31) return false;
+  const long long nodes = (long long)nx * ny;
+  const bool neq = precision == ISLBM_FP16NEQ;
+  const int w = neq ? YmGeom<Neq16, 2>::COLUMNS : YmGeom<float, 2>::COLUMNS;
+  const double f = (double)((nx + w - 1) / w * w) / ((nx + 63) / 64 * 64);
+  if (precision == ISLBM_FP32)
+    return nodes >= kYmMinNodes && f <= (nodes < kYmL2Nodes ? 1.15 : 1.3);
+  if (neq) return nodes >= kYmMinNodes && nx > 32 && f <= 1.2;
+  return nodes >= kYmMinNodes16 && nx > 32 && f <= 1.04;
 }
 
 // TMA boxes (x, y, planes) of a staged row pair: the populations, and the
@@ -706,7 +730,8 @@ struct YmBatch : BatchGroup {
 
 // Two steps of FP32 cavities in one launch.  *out stays null where single steps
 // (k_step_tma_batch) are the better choice: other storage forms, meshes below
-// the kernel's limits, or too few nodes to fill the GPU (step_2d_ym_takes).
+// the kernel's limits, too few nodes to fill the GPU (step_2d_ym_takes), or strips
+// and chunks that cost more than they save.
 cudaError_t make_batch_pair_group(const std::vector<Solver*>& members, int precision, int sms,
                                   cudaStream_t stream, BatchGroup** out) {
   *out = nullptr;
@@ -761,6 +786,16 @@ cudaError_t make_batch_pair_group(const std::vector<Solver*>& members, int preci
       best = rows;
     }
   }
+  // Rows that an SM's slot marches for one tile of a tile kernel's slot (two an
+  // SM): this kernel takes about 0.42 us for a row of `best_cost` (0.34 to 0.47 over
+  // 100 batches), the other 3.5 to 4.3 us for a tile while its two buffers are in
+  // L2 and 3.0 to 4.5 beyond (a step each).  Measured, batches of 64^2 to 768^2 (rows a tile, time of pairs over single
+  // steps): below 1.1M nodes 7.5-8.4 0.88-0.96, 8.7-9.8 1.02-1.21 (4 x 448^2 0.85),
+  // 10.2-14 1.10-1.43; above 7.4-8.9 0.70-0.95, 9.1-9.9 0.92-0.95, 10.1-12.6 0.97-1.09.
+  long long tiles = 0;
+  for (const Solver* m : members) tiles += (long long)((m->n[0] + 63) / 64) * ((m->n[1] + 7) / 8);
+  const double per_tile = nodes < kYmL2Nodes ? 8.5 : 10.0;
+  if (best_cost * 2 * sms > per_tile * (double)tiles) return cudaSuccess;
   std::vector<YmCav<float>> cavs(members.size());
   std::vector<YmBatchItem> items;
   for (size_t c = 0; c < members.size(); ++c) {
