@@ -150,7 +150,7 @@ struct YmGroup {
     ci = x - src0;
     bp = __float_as_int(a.w) - src0;
     bm = __float_as_int(b.w) - src0;
-    if (!(ISLBM_IN_WINDOW(ci, RS) && ISLBM_IN_WINDOW(bp, RS) && ISLBM_IN_WINDOW(bm, RS)))
+    if (!(ISLBM_IN_WINDOW(ci, RS) && ISLBM_IN_WINDOW(bp, RS - 2) && ISLBM_IN_WINDOW(bm, RS - 2)))
       ci = bp = bm = 0;
     wW = x == 0;
     wE = x == p.nx - 1;
@@ -322,7 +322,8 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, const CUtensorM
   [[maybe_unused]] auto decode = [&]() {
     if constexpr (G::NEQ) {
       const int x = x0 - NS + (int)threadIdx.x;
-      const int hc = x - xa, mc = x - ((x0 - NS) & ~3);
+      int hc = x - xa, mc = x - ((x0 - NS) & ~3);
+      if (!(ISLBM_IN_WINDOW(hc, G::TW) && ISLBM_IN_WINDOW(mc, G::MW))) hc = mc = 0;
       uint64_t* tfull = bars + 2 * DT;
       uint64_t* tempty = tfull + DR;
       float t0, ti;
@@ -405,7 +406,7 @@ __device__ __forceinline__ void ym_item(const CUtensorMap* tmap, const CUtensorM
       const int R = ya - 2 * (NS - s) - 1 + 2 * i;
       // tables of rows R - 1 and R, loaded before the wait, which hides their latency
       YmTables q{};
-      if (i > i0) {
+      if (i > i0 && ISLBM_IN_WINDOW(R - 1, p.ny) && ISLBM_IN_WINDOW(R, p.ny)) {
         q = YmTables{__ldg(tqp), __ldg(tqp + 1), __ldg(tqm), __ldg(tqm + 1)};
         tqp += 2;
         tqm += 2;
