@@ -1286,7 +1286,7 @@ extern "C" islbm_status islbm_cnn_forward(int stages, const int* channels, int b
     c.bias = static_cast<const float*>(params[5 + 2 * s]);
     c.out = acts[s + 1];
     c.act = up;
-    c.kchunk = gemm_kchunk((long long)batch * H * H, c.cout, up16(9 * c.cin), sms);
+    c.kchunk = chain_kchunk((long long)batch * H * H, c.cout, up16(9 * c.cin), c.cout % 8 == 0, sms);
     e = conv_forward(c, sms, st);
     if (e != cudaSuccess) return status_of(e);
   }
@@ -1361,7 +1361,7 @@ extern "C" islbm_status islbm_cnn_backward(int stages, const int* channels, int 
   }
   k_bias_sum<<<sum_first, 512, 0, st>>>(sums);
   const int n2 = base * base * channels[0];
-  const int dh_chunk = gemm_kchunk(batch, hidden, n2, sms), dh_tiles = (hidden + 7) / 8;
+  const int dh_chunk = chain_kchunk(batch, hidden, n2, n2 % 8 == 0, sms), dh_tiles = (hidden + 7) / 8;
   const int dh_x = (batch + kFcB - 1) / kFcB;
   // Warps of a tile: all 16 of a block, half of them at a time where there are
   // not as many chunks and the blocks still fill the GPU (a batch that fills it
