@@ -97,6 +97,15 @@ class WarmStartNet:
         self.fused = self.lib.islbm_cnn_backward_scratch(
             len(self.channels), self._chan, base, hidden, 1,
             ctypes.byref(ctypes.c_ulonglong())) == 0
+        # Batches: the fused layers' largest, and those in between that the chain takes
+        # sooner, images of one or two rows, of which the fused layers' tiles of 8 x 16
+        # pixels are nearly all padding.  Forward and backward over the chain's, networks
+        # of 1 to 2 rows and 16 or 64 channels: 4,096 samples 0.66-0.90, 16,384 1.01-1.72,
+        # 65,536 1.21-2.73 (3 rows 0.65-0.76, 0.79-0.90, 0.96-1.08).  The chain's grids
+        # end at 65,535 blocks of 64 pixels.
+        pixels = self.size ** 2
+        self._fused_most = (1 << 30) // pixels
+        self._chain_least, self._chain_most = (8192, 65535 * 64 // pixels) if pixels <= 4 else (0, 0)
         self.t = 0
         self.n_params = int(sum(int(np.prod(s)) for n, s in shapes
                                 if not n.startswith("Wc")) +
@@ -124,16 +133,11 @@ class WarmStartNet:
     # ---- forward ----
     def forward(self, z: np.ndarray, keep=True):
         """z: [B, 16] features.  Returns the output [B, S, S, 3] (torch, FP32)."""
-        B, pixels = z.shape[0], self.size ** 2
-        fused = self.fused and z.shape[1] == FEATURES and 1 <= B <= (1 << 30) // pixels
-        # Large batches of images of one or two rows: the fused layers' tiles of 8 x 16
-        # pixels are nearly all padding there.  Forward and backward over the chain's,
-        # networks of 1 to 2 rows and 16 or 64 channels: 4,096 samples 0.66-0.90, 16,384
-        # 1.01-1.72, 65,536 1.21-2.73 (3 rows 0.65-0.76, 0.79-0.90, 0.96-1.08).  The
-        # chain's grids end at 65,535 blocks of 64 pixels.
-        if fused and pixels <= 4 and 8192 < B <= 65535 * 64 // pixels:
-            fused = False
-        return self._forward_fused(z, keep) if fused else self._forward_chain(z, keep)
+        B = z.shape[0]
+        if (self.fused and z.shape[1] == FEATURES and 1 <= B <= self._fused_most
+                and not (self._chain_least < B <= self._chain_most)):
+            return self._forward_fused(z, keep)
+        return self._forward_chain(z, keep)
 
     def _forward_fused(self, z, keep):
         """forward() as fused layers, within the limits of islbm_cnn_forward."""
