@@ -855,7 +855,9 @@ __global__ void __launch_bounds__(512) k_fc_dh(const float* __restrict__ d2,
 // 16 samples and 3.8 times at 4,096.)  Chunks are blocks of their own; where
 // there are several, dw and db are their partial sums, which k_grad_sum adds.
 // A weight block takes 16 rows and 256 columns, a warp 32 of them, and reads
-// its fragments from global memory; a bias block takes 32 columns.
+// its fragments from global memory; a bias block takes 32 columns.  Bound by the
+// 4 MB that it writes and a launch's latency: 256 x 4096 weights of 16 samples 5.4
+// us, as scalar products 7.7.
 struct FcGrad {
   const float *a, *d;
   float *dw, *db;
