@@ -135,7 +135,9 @@ class WarmStartNet:
         """z: [B, 16] features.  Returns the output [B, S, S, 3] (torch, FP32)."""
         B = z.shape[0]
         if (self.fused and z.shape[1] == FEATURES and 1 <= B <= self._fused_most
-                and not (self._chain_least < B <= self._chain_most)):
+                and not (self._chain_least < B <= self._chain_most
+                         # (the chain's copy of the features cannot be captured)
+                         and not self.torch.cuda.is_current_stream_capturing())):
             return self._forward_fused(z, keep)
         return self._forward_chain(z, keep)
 

@@ -82,3 +82,18 @@ def test_tiny_images_in_large_batches_take_the_chain(base, channels, batch, fuse
     net = _net(base=base, channels=channels, hidden=16)
     net.forward(_z(batch))
     assert ("flat" in net.cache) == fused
+
+
+def test_tiny_images_in_a_captured_large_batch():
+    """A graph keeps the fused layers: the chain's copy of the features cannot be captured."""
+    import torch
+    net = _net(base=1, channels=(16,), hidden=16)
+    z = _z(9000)
+    net._forward_fused(z, False)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        y = net.forward(z, keep=False)
+    y.zero_()
+    g.replay()
+    assert torch.equal(y, net._forward_chain(z, False))
