@@ -442,9 +442,11 @@ ISLBM_API islbm_status islbm_cnn_adam(float* w, void* wb, const float* g, float*
  * convolves.  params: W1 [16][hidden], b1, W2 [hidden][base^2 channels[0]], b2,
  * then Wc_s [>= 9 channels[s]][channels[s + 1]], bc_s of every stage; weights
  * bf16, biases FP32.  z: batch x 16 features in HOST memory (read before the
- * call returns).  Written: zk [batch][16] (the features rounded to bf16; may be
- * NULL), h1 [batch][hidden], acts[0 .. stages]: the second layer's output and
- * every stage's.  acts 16-byte aligned.  Limits: 64 channels, 8 stages, 512
+ * call returns; above 1,920 samples, where zk is given and the stream is not
+ * being captured, the call waits for a copy of them).  Written: zk [batch][16]
+ * (the features rounded to bf16; may be NULL), h1 [batch][hidden], acts[0 ..
+ * stages]: the second layer's output and every stage's.  acts 16-byte aligned.
+ * Limits: 64 channels, 8 stages, 512
  * hidden units, 256 x 256 outputs (a wide layer fewer, by its shared memory),
  * 2^30 output pixels in a batch, and fewer than 2^27 images of 1 or 2 rows (the
  * weight gradient pads them to 16 pixels); ISLBM_ERR_ARG beyond them. */

@@ -779,8 +779,8 @@ __global__ void __launch_bounds__(128) k_fc_fwd(Fc p, const __grid_constant__ Z 
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int b = grp + (r >= 2 ? 8 : 0), n = n0 + warp * 16 + 8 * j + 2 * tig + (r & 1);
-        if (b < nb && n < p.n2) p.x0[(size_t)(bb + b) * p.n2 + n] =
-              tanhf(tot[j][r] + acc[j][r] + p.b2[n]);
+        if (b < nb && n < p.n2)
+          p.x0[(size_t)(bb + b) * p.n2 + n] = tanhf(tot[j][r] + acc[j][r] + p.b2[n]);
       }
     // (the next tile's features go to sz, read before the last barrier, and its
     // hidden layer to sh, behind the next one)
@@ -1247,8 +1247,11 @@ cudaError_t fc_forward(const Fc& f, const float* z, int sms, cudaStream_t st) {
   }
   if (f.B <= kZCopy || !f.zk || cap != cudaStreamCaptureStatusNone)
     return fc_launches<kZLarge>(f, z, sms, st);
-  const cudaError_t e =
+  cudaError_t e =
       cudaMemcpyAsync(f.zk, z, (size_t)f.B * kFeat * sizeof(float), cudaMemcpyHostToDevice, st);
+  // z may be freed once the call returns, and a copy from pageable memory need not
+  // have read it by then where the device reads the host's pages itself
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return e;
   k_round_features<<<(int)(((size_t)f.B * kFeat + 255) / 256), 256, 0, st>>>(f.zk,
                                                                             (size_t)f.B * kFeat);
